@@ -56,6 +56,12 @@ struct RwArgs {
   int me_only;  // evaluate pt[0] only and write me0 (no reductions)
   unsigned char* defer;  // mixed modes with a separate colour pass: its amplitude buffers, or null
   long long defer_ld;    // rows per amplitude plane (events rounded up to 128)
+  // Points whose coupling-stripped sum is the same (they differ in the overall
+  // coupling only) form one class: the distinct classes, in order of their
+  // first evaluation (class 0 holds evaluation 0)
+  int nkin;
+  short kin_rep[MAX_POINTS + 1];  // an evaluation of each class
+  short kin_of[MAX_POINTS + 1];   // each evaluation's class
   PointDev pt[MAX_POINTS + 1];  // [0] original, [1..P] modified points
 };
 
@@ -131,6 +137,52 @@ __device__ __forceinline__ double eval_point(const typename Proc::template mom_t
   else
     v = Proc::template me<R, LB>(q, pt, lane, gmask);
   return inside ? v : 0.0;
+}
+
+// The end of a reweighting launch: the block's warp sums sacc [nwarps][P+1] to
+// its partials, and in the last block to finish all partials to the results,
+// in a fixed order.
+__device__ __forceinline__ void reduce_sums(const RwArgs& a, const double2* sacc, unsigned long long nbad, double2* red,
+                                            int& is_last) {
+  const int stride = a.P + 1, tid = threadIdx.x, nw = blockDim.x >> 5;
+  __syncthreads();
+  for (int j = tid; j < stride; j += blockDim.x) {
+    double s = 0.0, c = 0.0;
+    for (int wi = 0; wi < nw; ++wi) two_sum_acc(s, c, sacc[wi * stride + j].x, sacc[wi * stride + j].y);
+    a.block_part[(long long)blockIdx.x * stride + j] = make_double2(s, c);
+  }
+  if (nbad) atomicAdd(a.nbad_count, nbad);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) is_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  for (int j = 0; j < stride; ++j) {
+    double s = 0.0, c = 0.0;
+    for (int b = tid; b < (int)gridDim.x; b += blockDim.x) {
+      const double2 v = __ldcg(a.block_part + (long long)b * stride + j);
+      two_sum_acc(s, c, v.x, v.y);
+    }
+    block_sum2(s, c, red);
+    if (tid == 0) {
+      if (a.sigma_acc) {  // chunked launches: carry (sum, compensation) in launch order
+        double2 t = a.accumulate ? a.sigma_acc[j] : make_double2(0.0, 0.0);
+        two_sum_acc(t.x, t.y, s, c);
+        a.sigma_acc[j] = t;
+        a.sigma[j] = t.x + t.y;
+        if (a.sigma_pair) a.sigma_pair[j] = t;
+      } else {
+        a.sigma[j] = s + c;
+        if (a.sigma_pair) a.sigma_pair[j] = make_double2(s, c);
+      }
+    }
+  }
+  if (tid == 0) {
+    const unsigned long long nb = atomicExch(a.nbad_count, 0ull);
+    *a.nbad_out = a.accumulate ? *a.nbad_out + nb : nb;
+    *a.ticket = 0u;
+  }
 }
 
 // MINB: resident blocks of 256 threads per SM the register allocation must
@@ -239,44 +291,7 @@ __global__ void __launch_bounds__(256, MINB) k_reweight(const __grid_constant__ 
       if (wl == 0) sacc[warp * stride + q] = make_double2(s, c);
     }
   }
-  __syncthreads();
-  for (int j = tid; j < stride; j += blockDim.x) {
-    double s = 0.0, c = 0.0;
-    for (int wi = 0; wi < nw; ++wi) two_sum_acc(s, c, sacc[wi * stride + j].x, sacc[wi * stride + j].y);
-    a.block_part[(long long)blockIdx.x * stride + j] = make_double2(s, c);
-  }
-  if (nbad) atomicAdd(a.nbad_count, nbad);
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) is_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  for (int j = 0; j < stride; ++j) {
-    double s = 0.0, c = 0.0;
-    for (int b = tid; b < (int)gridDim.x; b += blockDim.x) {
-      const double2 v = __ldcg(a.block_part + (long long)b * stride + j);
-      two_sum_acc(s, c, v.x, v.y);
-    }
-    block_sum2(s, c, red);
-    if (tid == 0) {
-      if (a.sigma_acc) {  // chunked launches: carry (sum, compensation) in launch order
-        double2 t = a.accumulate ? a.sigma_acc[j] : make_double2(0.0, 0.0);
-        two_sum_acc(t.x, t.y, s, c);
-        a.sigma_acc[j] = t;
-        a.sigma[j] = t.x + t.y;
-        if (a.sigma_pair) a.sigma_pair[j] = t;
-      } else {
-        a.sigma[j] = s + c;
-        if (a.sigma_pair) a.sigma_pair[j] = make_double2(s, c);
-      }
-    }
-  }
-  if (tid == 0) {
-    const unsigned long long nb = atomicExch(a.nbad_count, 0ull);
-    *a.nbad_out = a.accumulate ? *a.nbad_out + nb : nb;
-    *a.ticket = 0u;
-  }
+  reduce_sums(a, sacc, nbad, red, is_last);
 }
 
 // ---------------------------------------------------------------------------

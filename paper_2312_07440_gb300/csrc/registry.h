@@ -14,6 +14,7 @@ struct KernelEntry {
   int kind = 0;         // 0: k_reweight, 1: k_interp (interpolation surrogate), 2: k_amp_store
   int smem_per_thread = 0;  // dynamic shared memory of the amplitude code (bytes per thread)
   const void* func2 = nullptr;  // kind 2: the colour pass k_colour_tc<...>(RwArgs, int*)
+  int smem_per_warp_point = 16;  // dynamic shared memory per warp and evaluation (sums of the points)
 };
 
 // a k_reweight_multi instantiation: processes in its template order, each
@@ -45,6 +46,7 @@ void static_ee_5a(ProcStatic& s);
   void register_##name##_mixed(std::vector<KernelEntry>& t);
 void register_gg_ttgg_store_fp16(std::vector<KernelEntry>& t);
 void register_gg_ttgg_store_bf16(std::vector<KernelEntry>& t);
+void register_gg_ttgg_coop(std::vector<KernelEntry>& t);
 RW_DECLARE_QCD(gg_tt)
 RW_DECLARE_QCD(gg_ttg)
 RW_DECLARE_QCD(gg_ttgg)

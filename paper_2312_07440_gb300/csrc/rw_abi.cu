@@ -49,6 +49,7 @@ struct Registry {
     rw::register_gg_ttgg_fp64(kernels);
     rw::register_gg_ttgg_fp32(kernels);
     rw::static_gg_ttgg(st[RW_GG_TTGG]);
+    rw::register_gg_ttgg_coop(kernels);
     rw::register_ee_5a_fp64(kernels);
     rw::register_ee_5a_fp32(kernels);
     rw::static_ee_5a(st[RW_EE_5A]);
@@ -71,11 +72,15 @@ int default_lane_bits(int process, int mode) {
     case RW_EE_MUMU: return 2;
     case RW_GG_TT: return 0;
     case RW_GG_TTG: return 0;
-    case RW_GG_TTGG: return mode == RW_FP64 ? 1 : 2;
+    case RW_GG_TTGG: return 5;
     case RW_EE_5A: return 0;
   }
   return 0;
 }
+
+// lanes per event of the kernels that have no warp-per-event form (the
+// interpolation, the in-kernel tensor-core colour sum) when that is the choice
+int per_thread_lane_bits(int mode) { return mode == RW_FP64 ? 1 : 2; }
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -211,6 +216,28 @@ PointDev make_point(const rw_ctx* c, const rw_params& p, bool reshuffle) {
   return d;
 }
 
+// Evaluations with the same coupling-stripped sum (everything it depends on
+// equal: the top mass for the QCD processes, nothing for the photons), as
+// classes in order of their first evaluation.
+void classify(const rw_ctx* c, RwArgs& a) {
+  auto same = [c](const PointDev& x, const PointDev& y) {
+    if (c->process == RW_EE_5A) return true;
+    if (c->process == RW_EE_MUMU)
+      return x.e == y.e && x.gL == y.gL && x.gR == y.gR && x.MZ == y.MZ && x.WZ == y.WZ;
+    return x.m_t == y.m_t && x.reshuffle == y.reshuffle;
+  };
+  a.nkin = 0;
+  for (int j = 0; j <= a.P; ++j) {
+    int k = a.nkin;  // newest class first: scans often list equal points in a row
+    while (k > 0 && !same(a.pt[j], a.pt[a.kin_rep[k - 1]])) --k;
+    if (k == 0) {
+      a.kin_rep[a.nkin] = (short)j;
+      k = ++a.nkin;
+    }
+    a.kin_of[j] = (short)(k - 1);
+  }
+}
+
 // workspace: 256-B header (ticket, bad-event counter; sigma [P+1] and the
 // bad-event count from byte 64), block partials double2 [GRID_CAP][P+1], then
 // the results' (sum, compensation) pairs double2 [P+1]
@@ -290,13 +317,30 @@ struct Shape {
   size_t smem;
 };
 
-int shape(rw_ctx* c, int P, Shape& sh) {
+// lanes per event (2^bits) of the context's kernel of a kind; a choice that
+// kind was not compiled for falls back to a per-thread one
+int lane_bits_for(const rw_ctx* c, int kind) {
   const int lb = c->lane_bits >= 0 ? c->lane_bits : default_lane_bits(c->process, c->mode);
+  return lb < 5 || registry().find(c->process, c->mode, lb, kind) ? lb : per_thread_lane_bits(c->mode);
+}
+
+// Threads per block: the caller's choice, else 128.  The warp-per-event kernels
+// (32 lanes) run 8 warps per block, so that the shared memory left beside the
+// task tables holds the most warps an SM can have, unless there are too few
+// events to give every SM that many: then 2, which spreads them over the SMs.
+int block_for(const rw_ctx* c, int lb, long long E) {
+  if (c->block > 0) return c->block;
+  if (lb < 5) return 128;
+  return E >= 16LL * c->sm_count ? 256 : 64;
+}
+
+int shape(rw_ctx* c, int P, long long E, Shape& sh) {
+  const int lb = lane_bits_for(c, 0);
   const KernelEntry* k = registry().find(c->process, c->mode, lb);
   if (!k) return fail(c, RW_ERR_MODE, "no kernel for process %d mode %d lane_bits %d", c->process, c->mode, lb);
-  const int block = c->block > 0 ? c->block : 128;
+  const int block = block_for(c, lb, E);
   if (block > k->max_block) return fail(c, RW_ERR_ARG, "block %d above this variant's %d", block, k->max_block);
-  const size_t smem = (size_t)k->smem_per_thread * block + (size_t)(block / 32) * (P + 1) * sizeof(double2);
+  const size_t smem = (size_t)k->smem_per_thread * block + (size_t)(block / 32) * (P + 1) * k->smem_per_warp_point;
   const size_t smem_total = smem + static_smem(k->func);
   if (c->smem_optin > 0 && smem_total > (size_t)c->smem_optin)
     return fail(c, RW_ERR_ARG,
@@ -322,10 +366,10 @@ int shape(rw_ctx* c, int P, Shape& sh) {
 
 // the amplitude pass, then the tensor-core colour pass (colour_tc.cuh)
 int launch_deferred(rw_ctx* c, RwArgs& a, const KernelEntry* d) {
-  const int block = c->block > 0 ? c->block : 128;
+  const int block = block_for(c, d->lane_bits, a.E);
   const int lanes = 1 << d->lane_bits;
   if (block > d->max_block || lanes > block) return fail(c, RW_ERR_ARG, "block %d does not fit this variant", block);
-  const size_t smem = (size_t)d->smem_per_thread * block;
+  const size_t smem = (size_t)d->smem_per_thread * block;  // no sums in this pass
   const size_t smem_total = smem + static_smem(d->func);
   if (c->smem_optin > 0 && smem_total > (size_t)c->smem_optin)
     return fail(c, RW_ERR_ARG, "block %d needs %zu bytes of shared memory (%d per thread), more than the %d a block may have",
@@ -380,12 +424,13 @@ int launch_deferred(rw_ctx* c, RwArgs& a, const KernelEntry* d) {
 
 int launch(rw_ctx* c, RwArgs& a) {
   c->deferred_last = false;
+  if (!a.me_only) classify(c, a);
   if (a.defer) {
     const int lb = c->lane_bits >= 0 ? c->lane_bits : default_lane_bits(c->process, c->mode);
     if (const KernelEntry* d = registry().find(c->process, c->mode, lb, 2)) return launch_deferred(c, a, d);
   }
   Shape sh;
-  int rc = shape(c, a.P, sh);
+  int rc = shape(c, a.P, a.E, sh);
   if (rc) return rc;
   const KernelEntry* k = sh.k;
   const int block = sh.block, lanes = sh.lanes, per_sm = sh.per_sm;
@@ -556,9 +601,9 @@ int rw_set_tuning(rw_ctx* c, int lane_bits, int block) {
     return fail(c, RW_ERR_ARG, "block must be a multiple of 32 in [32, 256]");
   if (lane_bits >= 0 && c->process >= 0) {
     const KernelEntry* k = registry().find(c->process, c->mode, lane_bits);
-    if (!k) return fail(c, RW_ERR_MODE, "lane_bits %d not compiled for this process/mode", lane_bits);
     const KernelEntry* d = registry().find(c->process, c->mode, lane_bits, 2);  // separate colour pass
-    const int max_block = d ? std::max(k->max_block, d->max_block) : k->max_block;
+    if (!k && !d) return fail(c, RW_ERR_MODE, "lane_bits %d not compiled for this process/mode", lane_bits);
+    const int max_block = std::max(k ? k->max_block : 0, d ? d->max_block : 0);
     if (block > max_block) return fail(c, RW_ERR_ARG, "block above this variant's %d", max_block);
     if ((1 << lane_bits) > (block ? block : 128)) return fail(c, RW_ERR_ARG, "more lanes than threads");
   }
@@ -571,7 +616,7 @@ int rw_get_tuning(const rw_ctx* c, int* lane_bits, int* block) {
   if (!c || !lane_bits || !block) return RW_ERR_NULL;
   if (c->process < 0) return RW_ERR_STATE;
   *lane_bits = c->lane_bits >= 0 ? c->lane_bits : default_lane_bits(c->process, c->mode);
-  *block = c->block > 0 ? c->block : 128;
+  *block = block_for(c, *lane_bits, c->mom ? c->E : int64_t(1) << 40);
   return RW_OK;
 }
 
@@ -598,7 +643,8 @@ int rw_autotune(rw_ctx* c, int64_t max_events, const char* cache_path, double* m
         double ms;
         if (sscanf(line, "{\"key\": \"%511[^\"]\", \"lane_bits\": %d, \"block\": %d, \"ms\": %lf}", k, &lb, &bl, &ms) ==
                 4 &&
-            strcmp(k, key) == 0 && registry().find(c->process, c->mode, lb)) {
+            strcmp(k, key) == 0 &&
+            (registry().find(c->process, c->mode, lb) || registry().find(c->process, c->mode, lb, 2))) {
           fclose(f);
           c->lane_bits = lb;
           c->block = bl;
@@ -619,12 +665,15 @@ int rw_autotune(rw_ctx* c, int64_t max_events, const char* cache_path, double* m
   int best_lb = -1, best_bl = 0;
   static const int blocks[] = {64, 128, 256};
   for (const auto& k : registry().kernels) {
-    if (k.process != c->process || k.mode != c->mode || k.kind != 0) continue;
-    // with the separate colour pass attached, its amplitude kernel's limit
-    const KernelEntry* d = registry().find(c->process, c->mode, k.lane_bits, 2);
+    if (k.process != c->process || k.mode != c->mode || k.kind == 1) continue;
     RwArgs probe{};
     probe.P = (int)c->pts.size();
     set_defer(c, probe, probe.P + 1);
+    // amplitude passes of the separate colour sum run under the lanes of the
+    // fused variant, or by themselves where there is none
+    if (k.kind == 2 && (!probe.defer || registry().find(c->process, c->mode, k.lane_bits))) continue;
+    // with the separate colour pass attached, its amplitude kernel's limit
+    const KernelEntry* d = registry().find(c->process, c->mode, k.lane_bits, 2);
     const int max_block = (d && probe.defer) ? d->max_block : k.max_block;
     for (int bl : blocks) {
       if ((1 << k.lane_bits) > bl || bl > max_block) continue;
@@ -849,7 +898,7 @@ int rw_reweight_host(rw_ctx* c, const double* h_mom, const double* h_w, int64_t 
   int rc = load_events(c, d_mom, d_w, E, d_ws, ws_bytes, true);
   if (rc) return rc;
   Shape sh;
-  if ((rc = shape(c, P, sh))) return rc;
+  if ((rc = shape(c, P, E, sh))) return rc;
   // events one launch keeps resident, and the chunk size: about E/8, rounded
   // up to it; the first chunk is one resident set only (its copy-in is the
   // part of the transfer nothing overlaps)
@@ -997,12 +1046,12 @@ extern "C" int rw_reweight_noalloc(rw_ctx* c, const double* d_mom, const double*
   char* scratch = static_cast<char*>(noalloc_scratch(c->device));
   if (!scratch) return noalloc_fail(c, RW_ERR_CUDA, "scratch lookup");
 
-  const int lb = c->lane_bits >= 0 ? c->lane_bits : default_lane_bits(c->process, c->mode);
+  const int lb = lane_bits_for(c, 0);
   const KernelEntry* k = registry().find(c->process, c->mode, lb);
   if (!k) return noalloc_fail(c, RW_ERR_MODE, "no kernel");
-  const int block = c->block > 0 ? c->block : 128;
+  const int block = block_for(c, lb, E);
   if (block > k->max_block) return noalloc_fail(c, RW_ERR_ARG, "block too large");
-  const size_t smem = (size_t)k->smem_per_thread * block + (size_t)(block / 32) * (P + 1) * sizeof(double2);
+  const size_t smem = (size_t)k->smem_per_thread * block + (size_t)(block / 32) * (P + 1) * k->smem_per_warp_point;
   if (c->smem_optin > 0 && smem + static_smem(k->func) > (size_t)c->smem_optin)
     return noalloc_fail(c, RW_ERR_ARG, "block too large");
   if (ensure_smem(k->func, smem) != cudaSuccess) {
@@ -1033,6 +1082,7 @@ extern "C" int rw_reweight_noalloc(rw_ctx* c, const double* d_mom, const double*
     const bool moved = moves_event(c, c->pts[j]);
     a.pt[1 + j] = make_point(c, c->pts[j], moved);
   }
+  classify(c, a);
   a.ticket = reinterpret_cast<unsigned int*>(scratch);
   a.nbad_count = reinterpret_cast<unsigned long long*>(scratch + 8);
   a.block_part = reinterpret_cast<double2*>(scratch + NOALLOC_HEADER);
@@ -1567,7 +1617,7 @@ int rw_reweight_interp(rw_ctx* c, int n_nodes, double tol, double* d_wnew, unsig
   if (ws_bytes < L.total) return fail(c, RW_ERR_WORKSPACE, "workspace %zu < %zu", ws_bytes, L.total);
   const int axis = interp_axis(c);
   if (axis < 0) return fail(c, RW_ERR_ARG, "the points must differ from the original parameters in one field only");
-  const int lb = c->lane_bits >= 0 ? c->lane_bits : default_lane_bits(c->process, c->mode);
+  const int lb = lane_bits_for(c, 1);
   const KernelEntry* k = registry().find(c->process, c->mode, lb, 1);
   if (!k) return fail(c, RW_ERR_MODE, "no interpolation kernel for process %d mode %d lane_bits %d", c->process,
                       c->mode, lb);
@@ -1611,19 +1661,22 @@ int rw_reweight_interp(rw_ctx* c, int n_nodes, double tol, double* d_wnew, unsig
   cudaError_t e = cudaMemsetAsync(ia.counts, 0, 16, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "memset");
   {
-    Shape sh;
-    if ((rc = shape(c, 0, sh))) return rc;
-    const size_t ismem = (size_t)k->smem_per_thread * sh.block;
+    const int block = block_for(c, lb, E);
+    if (block > k->max_block) return fail(c, RW_ERR_ARG, "block %d above this variant's %d", block, k->max_block);
+    const size_t ismem = (size_t)k->smem_per_thread * block;
+    if (c->smem_optin > 0 && ismem + static_smem(k->func) > (size_t)c->smem_optin)
+      return fail(c, RW_ERR_ARG, "block %d needs %zu bytes of shared memory, more than the %d a block may have", block,
+                  ismem, c->smem_optin);
     if ((e = ensure_smem(k->func, ismem)) != cudaSuccess)
       return cuda_fail(c, e, "cudaFuncSetAttribute(MaxDynamicSharedMemorySize)");
     int per_sm = 1;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k->func, sh.block, ismem)) != cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k->func, block, ismem)) != cudaSuccess)
       return cuda_fail(c, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    const long long need = (E * (1 << lb) + sh.block - 1) / sh.block;
+    const long long need = (E * (1 << lb) + block - 1) / block;
     const int grid = (int)std::max(1LL, std::min<long long>({(long long)GRID_CAP,
                                                               (long long)std::max(1, per_sm) * c->sm_count, need}));
     void* args[] = {&ia};
-    if ((e = cudaLaunchKernel(k->func, dim3(grid), dim3(sh.block), args, ismem, c->stream)) != cudaSuccess)
+    if ((e = cudaLaunchKernel(k->func, dim3(grid), dim3(block), args, ismem, c->stream)) != cudaSuccess)
       return cuda_fail(c, e, "interpolation kernel launch");
   }
   if ((e = cudaMemcpyAsync(c->h_stage, ia.counts, 16, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess ||
