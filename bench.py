@@ -314,12 +314,24 @@ def measured_peaks(dev_index, stream_handle):
     return out
 
 
-def alu_roofline(info, E, P, t_step, mode, peaks, workload):
+def evaluations(process, pts):
+    """Helicity sums per event of a launch: points that differ from an earlier
+    one (or the original) only in the overall coupling share its sum."""
+    if process == "ee_5a":
+        return 1
+    p0 = ev.param_vector()
+    if process == "ee_mumu":
+        return len({tuple(q[4:]) for q in [p0, *pts]})
+    return len({float(q[1]) for q in [p0, *pts]})
+
+
+def alu_roofline(info, E, pts, t_step, mode, peaks, workload):
     """Roofline of the fused kernel against the plain-ALU pipe it is bound by:
-    algorithmic flops = (1 + P) x the generator's static count of one helicity
-    sum per event; the ncu-executed count beside it when a profile of the
-    current sources records one."""
-    flops_event = (1 + P) * info.flops_hel_sum
+    algorithmic flops = the launch's distinct evaluations x the generator's
+    static count of one helicity sum per event; the ncu-executed count beside
+    it when a profile of the current sources records one."""
+    P = len(pts)
+    flops_event = evaluations(ev.WORKLOADS[workload].process, pts) * info.flops_hel_sum
     achieved = E * flops_event / t_step / 1e12
     pipe = "fp64" if mode == "fp64" else "fp32"
     peak = peaks[pipe]
@@ -487,7 +499,7 @@ def run_ours(args):
     if not args.no_e2e:
         e2e = run_e2e(ctx, torch, dev, mom_h, w_h, E, P, N, world, args)
     info = rwgt.process_info(wl.process)
-    roof = alu_roofline(info, E, P, t_step, args.mode, peaks, wl.name)
+    roof = alu_roofline(info, E, pts, t_step, args.mode, peaks, wl.name)
     ctx.close()
     del ws
 
@@ -571,7 +583,7 @@ def run_variant(torch, rwgt, dev, stream, wl, variant, mode, sample, args, flush
            "point_set": f"{variant}: {POINT_SETS.get(variant, variant)}", "mode": mode,
            "value": E * P / t, "unit": UNIT, "ms_per_step": 1e3 * t, "dtype": DTYPE[mode],
            "tuning": {"lane_bits": lb, "block": bl},
-           "roofline": alu_roofline(info, E, P, t, mode, peaks, wl.name),
+           "roofline": alu_roofline(info, E, pts, t, mode, peaks, wl.name),
            "accuracy_vs_oracle": accuracy_sample(wl, pts, mom_h, w_h, wn, mode, n=n_acc, variant=variant)}
     if variant == "default" and wl.process in ("gg_ttg", "gg_ttgg"):
         out["r_is_exactly_one"] = bool(torch.all(wn == w.unsqueeze(0)).item())

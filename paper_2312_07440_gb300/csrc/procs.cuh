@@ -1,4 +1,4 @@
-// Process adapters for the fused kernel: |M|^2 of one event for one
+// Process adapters for the fused kernel: |M|^2 / cscale of one event for one
 // parameter point, helicity slices combined across the 2^LB lanes of a group.
 #pragma once
 #include <type_traits>
@@ -83,7 +83,7 @@ struct QcdProc {
     }
 #pragma unroll
     for (int o = 1; o < (1 << LB); o <<= 1) s += __shfl_xor_sync(gmask, s, o);
-    return s * pt.cscale;
+    return s;
   }  // Out of line by default: every evaluation runs the same instructions, so
   // identical inputs give bitwise identical |M|^2 (r == 1 exactly for
   // unchanged parameters).  Inlined (Tag::INLINE_ME, FP32) the kernel's one
@@ -146,7 +146,7 @@ struct QcdProc {
 };
 
 // e-(p0) e+(p1) -> n photons (massless QED).  Tag provides NA, NEXT, MAX_LB
-// and hel_sum<R, LB>() (generated by gen/qed_gen.py); |M|^2 = cscale * sum,
+// and hel_sum<R, LB>() (generated by gen/qed_gen.py); |M|^2 = cscale * sum (the caller's product),
 // cscale = e^(2n) / (4 n!).  Nothing moves with the parameters (no reshuffle).
 template <class Tag>
 struct QedProc {
@@ -173,7 +173,7 @@ struct QedProc {
     double s = double(Tag::template hel_sum<R, LB>(X, Kn, lane));
 #pragma unroll
     for (int o = 1; o < (1 << LB); o <<= 1) s += __shfl_xor_sync(gmask, s, o);
-    return s * pt.cscale;
+    return s;
   }
   template <class R>
   __device__ __forceinline__ static bool reshuffle(const mom_t<R> (&p)[NEXT][4], double, mom_t<R> (&q)[NEXT][4]) {

@@ -236,6 +236,13 @@ void classify(const rw_ctx* c, RwArgs& a) {
     }
     a.kin_of[j] = (short)(k - 1);
   }
+  int n[rw::MAX_POINTS + 1] = {};
+  for (int j = 0; j <= a.P; ++j) ++n[a.kin_of[j]];
+  for (int k = 0, at = 0; k < a.nkin; ++k) {
+    a.kin_end[k] = (short)at;  // where the class begins, until its evaluations are placed
+    at += n[k];
+  }
+  for (int j = 0; j <= a.P; ++j) a.order[a.kin_end[a.kin_of[j]]++] = (short)j;
 }
 
 // workspace: 256-B header (ticket, bad-event counter; sigma [P+1] and the
