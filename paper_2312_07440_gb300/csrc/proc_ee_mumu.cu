@@ -7,10 +7,10 @@
 namespace rw {
 
 // Floating-point operations of EeMumu::me's helicity sum as written, per
-// helicity: 4 fermion currents (4 x 72), the vector and axial sums (16 + 48),
-// the Z exchange (dot 30, two real-complex products 28, 6 + 2 + 2), the photon
-// exchange (dot 30, 2), their sum (6 + 2), |M|^2 and its accumulation (4).
-constexpr long long EE_MUMU_FLOPS_HEL_SUM = EeMumu::NHEL * 464LL;
+// chirality configuration: 2 currents (2 x 32), their products with each other
+// and with k (30 + 2 x 14), the Z exchange (12), the photon exchange and the
+// sum (10), |M|^2 and its accumulation (4), g (1).
+constexpr long long EE_MUMU_FLOPS_HEL_SUM = 4 * 149LL;
 
 void register_ee_mumu(std::vector<KernelEntry>& t, ProcStatic& s) {
   s = {4, 16, 1, 2, 1, 1, 0, EE_MUMU_FLOPS_HEL_SUM, 4};
