@@ -134,12 +134,12 @@ struct QcdProc {
     return inside;
   }
 
-  // FP64 mode refines the FP32 Newton solution with two FP64 steps, the FP32
-  // modes with one double-float step.
+  // FP64 mode refines the FP32 Newton solution with one third-order FP64 step,
+  // the FP32 modes with one double-float step.
   template <class R>
   __device__ __forceinline__ static bool reshuffle(const mom_t<R> (&p)[NEXT][4], double mt, mom_t<R> (&q)[NEXT][4]) {
     if constexpr (sizeof(R) == 8)
-      return reshuffle_tops<NEXT, 2>(p, mt, q);
+      return reshuffle_tops<NEXT>(p, mt, q);
     else
       return reshuffle_tops<NEXT>(p, mt, q);
   }

@@ -64,17 +64,6 @@ struct Acc<float> {
   using two = df;
 };
 
-__device__ __forceinline__ void comp_add(double& s, double& c, double hi, double lo) {
-  const dd t = dd_two_sum(s, hi);
-  s = t.hi;
-  c += t.lo + lo;
-}
-__device__ __forceinline__ void comp_add(float& s, float& c, float hi, float lo) {
-  const df t = df_two_sum(s, hi);
-  s = t.hi;
-  c = __fadd_rn(c, __fadd_rn(t.lo, lo));
-}
-
 constexpr int NBATCH = 2;  // evaluations a warp carries at a time
 
 // Objects (complex 4-vectors and spinors), indices within one evaluation ...
