@@ -12,7 +12,7 @@ constexpr int K = 6;
 constexpr int NHEL = 32;
 constexpr int NDIAG = 16;
 constexpr int MAX_LB = 3;  // helicity levels that can be spread over lanes
-constexpr int NJS = 3;  // currents of 3+ gluons, one JStore slot each
+constexpr int NJS = 0;  // currents of 3+ gluons, one JStore slot each
 constexpr int CDEN = 9;
 constexpr int IDENT = 1;  // identical outgoing gluons (1/IDENT!)
 constexpr unsigned OUTGOING_GLUONS = 4u;  // bit g: gluon g outgoing
@@ -38,6 +38,8 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
     const int h0 = 0;
     const cv<R> E0 = h0 ? X.eps[0][1] : X.eps[0][0];
     const ws<R> W0 = weyl_form(E0);
+    const sp<R> T0_0 = row_prop(Kn.qc[6], Kn.mc[6], row_slash(W0, X.ub[0]));
+    const sp<R> T0_1 = row_prop(Kn.qc[6], Kn.mc[6], row_slash(W0, X.ub[1]));
     [[maybe_unused]] sp<R> S_0v0, S_0v1;
     if constexpr (LB < 3) {
       S_0v0 = fprop(Kn.qc[1], Kn.mc[1], slash(W0, X.v[0]));
@@ -48,6 +50,8 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
       const int h1 = LB >= 1 ? ((lane >> (LB - 1)) & 1) : i1;
       const cv<R> E1 = h1 ? X.eps[1][1] : X.eps[1][0];
       const ws<R> W1 = weyl_form(E1);
+      const sp<R> T1_0 = row_prop(Kn.qc[5], Kn.mc[5], row_slash(W1, X.ub[0]));
+      const sp<R> T1_1 = row_prop(Kn.qc[5], Kn.mc[5], row_slash(W1, X.ub[1]));
       cv<R> J0_1 = vvv(E0, Kn.P[1], E1, Kn.P[2], Kn.cg[3]);
       const cv<R> J1_0 = neg(J0_1);
       #pragma unroll 1
@@ -55,106 +59,103 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
         const int h2 = LB >= 2 ? ((lane >> (LB - 2)) & 1) : i2;
         const cv<R> E2 = h2 ? X.eps[2][1] : X.eps[2][0];
         const ws<R> W2 = weyl_form(E2);
+        const sp<R> T2_0 = row_prop(Kn.qc[3], Kn.mc[3], row_slash(W2, X.ub[0]));
+        const sp<R> T2_1 = row_prop(Kn.qc[3], Kn.mc[3], row_slash(W2, X.ub[1]));
         cv<R> J0_2 = vvv(E0, Kn.P[1], E2, Kn.P[4], Kn.cg[5]);
         cv<R> J1_2 = vvv(E1, Kn.P[2], E2, Kn.P[4], Kn.cg[6]);
         const cv<R> J2_0 = neg(J0_2);
         const cv<R> J2_1 = neg(J1_2);
-        cv<R> J0_1_2 = vvv(E0, Kn.P[1], J1_2, Kn.P[6], Kn.cg[7]);
-        vvv_acc(J0_1_2, J0_1, Kn.P[3], E2, Kn.P[4], Kn.cg[7]);
-        vvvv_acc(J0_1_2, E0, E1, E2, Kn.c4[7]);
-        js.put(0, J0_1_2);
-        cv<R> J0_2_1 = vvv(E0, Kn.P[1], J2_1, Kn.P[6], Kn.cg[7]);
-        vvv_acc(J0_2_1, J0_2, Kn.P[5], E1, Kn.P[2], Kn.cg[7]);
-        vvvv_acc(J0_2_1, E0, E2, E1, Kn.c4[7]);
-        js.put(1, J0_2_1);
-        cv<R> J1_0_2 = vvv(E1, Kn.P[2], J0_2, Kn.P[5], Kn.cg[7]);
-        vvv_acc(J1_0_2, J1_0, Kn.P[3], E2, Kn.P[4], Kn.cg[7]);
-        vvvv_acc(J1_0_2, E1, E0, E2, Kn.c4[7]);
-        js.put(2, J1_0_2);
+        const cv<R> J0_1_2 = current3(E0, E1, E2, J0_1, J1_2, Kn.P[1], Kn.P[4], Kn.P[3], Kn.P[6], Kn.cg[7]);
+        const cv<R> J0_2_1 = current3(E0, E2, E1, J0_2, J2_1, Kn.P[1], Kn.P[2], Kn.P[5], Kn.P[6], Kn.cg[7]);
+        const cv<R> J1_2_0 = J0_2_1;
+        const cv<R> J2_1_0 = J0_1_2;
         #pragma unroll 1
         for (int i3 = 0; i3 < (LB >= 3 ? 1 : 2); ++i3) {
           const int h3 = LB >= 3 ? ((lane >> (LB - 3)) & 1) : i3;
           const sp<R> S_E = h3 ? X.v[1] : X.v[0];
-          constexpr bool SH = sizeof(R) == 8;  // share every repeated slash (FP64)
           sp<R> S_0;
           if constexpr (LB < 3) S_0 = h3 ? S_0v1 : S_0v0;
           else S_0 = fprop(Kn.qc[1], Kn.mc[1], slash(W0, S_E));
-          sp<R> tS_1_0;
-          [[maybe_unused]] sp<R> Y0_1__E;  // Jslash(0,1) psi(E)
-          if constexpr (true) Y0_1__E = slash(J0_1, S_E);
-          if constexpr (true) tS_1_0 = spneg(Y0_1__E); else tS_1_0 = slash(J1_0, S_E);
-          slash_acc(tS_1_0, W1, S_0);  // single-gluon term, fused
-          const sp<R> S_1_0 = fprop(Kn.qc[3], Kn.mc[3], tS_1_0);
-          sp<R> X5;
-          [[maybe_unused]] sp<R> Y1_2__0;  // Jslash(1,2) psi(0)
-          [[maybe_unused]] sp<R> Y0_1_2__E;  // Jslash(0,1,2) psi(E)
-          if constexpr (true) Y1_2__0 = slash(J1_2, S_0);
-          if constexpr (true) X5 = spneg(Y1_2__0); else X5 = slash(J2_1, S_0);
-          if constexpr (SH) Y0_1_2__E = slash(js.get(0), S_E);
-          if constexpr (SH) spadd(X5, Y0_1_2__E); else slash_acc(X5, js.get(0), S_E);
-          slash_acc(X5, W2, S_1_0);  // single-gluon term, fused
-          const cx<R> A5_0 = rowcol(X.ub[0], X5), A5_1 = rowcol(X.ub[1], X5);
-          sp<R> tS_2_0;
-          [[maybe_unused]] sp<R> Y0_2__E;  // Jslash(0,2) psi(E)
-          if constexpr (true) Y0_2__E = slash(J0_2, S_E);
-          if constexpr (true) tS_2_0 = spneg(Y0_2__E); else tS_2_0 = slash(J2_0, S_E);
-          slash_acc(tS_2_0, W2, S_0);  // single-gluon term, fused
-          const sp<R> S_2_0 = fprop(Kn.qc[5], Kn.mc[5], tS_2_0);
-          sp<R> X3;
-          [[maybe_unused]] sp<R> Y0_2_1__E;  // Jslash(0,2,1) psi(E)
-          if constexpr (true) X3 = Y1_2__0; else X3 = slash(J1_2, S_0);
-          if constexpr (true) Y0_2_1__E = slash(js.get(1), S_E);
-          if constexpr (true) spadd(X3, Y0_2_1__E); else slash_acc(X3, js.get(1), S_E);
-          slash_acc(X3, W1, S_2_0);  // single-gluon term, fused
-          const cx<R> A3_0 = rowcol(X.ub[0], X3), A3_1 = rowcol(X.ub[1], X3);
-          sp<R> tS_1 = slash(W1, S_E);
-          const sp<R> S_1 = fprop(Kn.qc[2], Kn.mc[2], tS_1);
-          sp<R> tS_0_1;
-          if constexpr (true) tS_0_1 = Y0_1__E; else tS_0_1 = slash(J0_1, S_E);
-          slash_acc(tS_0_1, W0, S_1);  // single-gluon term, fused
-          const sp<R> S_0_1 = fprop(Kn.qc[3], Kn.mc[3], tS_0_1);
-          sp<R> X4;
-          [[maybe_unused]] sp<R> Y0_2__1;  // Jslash(0,2) psi(1)
-          [[maybe_unused]] sp<R> Y1_0_2__E;  // Jslash(1,0,2) psi(E)
-          if constexpr (true) Y0_2__1 = slash(J0_2, S_1);
-          if constexpr (true) X4 = spneg(Y0_2__1); else X4 = slash(J2_0, S_1);
-          if constexpr (true) Y1_0_2__E = slash(js.get(2), S_E);
-          if constexpr (true) spadd(X4, Y1_0_2__E); else slash_acc(X4, js.get(2), S_E);
-          slash_acc(X4, W2, S_0_1);  // single-gluon term, fused
-          const cx<R> A4_0 = rowcol(X.ub[0], X4), A4_1 = rowcol(X.ub[1], X4);
-          sp<R> tS_2_1;
-          [[maybe_unused]] sp<R> Y1_2__E;  // Jslash(1,2) psi(E)
-          if constexpr (true) Y1_2__E = slash(J1_2, S_E);
-          if constexpr (true) tS_2_1 = spneg(Y1_2__E); else tS_2_1 = slash(J2_1, S_E);
-          slash_acc(tS_2_1, W2, S_1);  // single-gluon term, fused
-          const sp<R> S_2_1 = fprop(Kn.qc[6], Kn.mc[6], tS_2_1);
-          sp<R> X1;
-          if constexpr (true) X1 = Y0_2__1; else X1 = slash(J0_2, S_1);
-          if constexpr (true) spadd(X1, Y0_2_1__E); else slash_acc(X1, js.get(1), S_E);
-          slash_acc(X1, W0, S_2_1);  // single-gluon term, fused
-          const cx<R> A1_0 = rowcol(X.ub[0], X1), A1_1 = rowcol(X.ub[1], X1);
-          sp<R> tS_2 = slash(W2, S_E);
-          const sp<R> S_2 = fprop(Kn.qc[4], Kn.mc[4], tS_2);
-          sp<R> tS_0_2;
-          if constexpr (true) tS_0_2 = Y0_2__E; else tS_0_2 = slash(J0_2, S_E);
-          slash_acc(tS_0_2, W0, S_2);  // single-gluon term, fused
-          const sp<R> S_0_2 = fprop(Kn.qc[5], Kn.mc[5], tS_0_2);
-          sp<R> X2;
-          [[maybe_unused]] sp<R> Y0_1__2;  // Jslash(0,1) psi(2)
-          if constexpr (true) Y0_1__2 = slash(J0_1, S_2);
-          if constexpr (true) X2 = spneg(Y0_1__2); else X2 = slash(J1_0, S_2);
-          if constexpr (true) spadd(X2, Y1_0_2__E); else slash_acc(X2, js.get(2), S_E);
-          slash_acc(X2, W1, S_0_2);  // single-gluon term, fused
-          const cx<R> A2_0 = rowcol(X.ub[0], X2), A2_1 = rowcol(X.ub[1], X2);
-          sp<R> tS_1_2;
-          if constexpr (true) tS_1_2 = Y1_2__E; else tS_1_2 = slash(J1_2, S_E);
-          slash_acc(tS_1_2, W1, S_2);  // single-gluon term, fused
-          const sp<R> S_1_2 = fprop(Kn.qc[6], Kn.mc[6], tS_1_2);
-          sp<R> X0;
-          if constexpr (true) X0 = Y0_1__2; else X0 = slash(J0_1, S_2);
-          if constexpr (SH) spadd(X0, Y0_1_2__E); else slash_acc(X0, js.get(0), S_E);
-          slash_acc(X0, W0, S_1_2);  // single-gluon term, fused
-          const cx<R> A0_0 = rowcol(X.ub[0], X0), A0_1 = rowcol(X.ub[1], X0);
+          const sp<R> S_1 = fprop(Kn.qc[2], Kn.mc[2], slash(W1, S_E));
+          const sp<R> S_2 = fprop(Kn.qc[4], Kn.mc[4], slash(W2, S_E));
+          cx<R> A0_0, A0_1, A1_0, A1_1, A2_0, A2_1, A3_0, A3_1, A4_0, A4_1, A5_0, A5_1;
+          {
+            const ws<R> WJ = weyl_form(J0_1);
+            sp<R> x = slash(WJ, S_E), y = spneg(x);  // J(01) v and J(10) v
+            slash_acc(x, W0, S_1);
+            slash_acc(y, W1, S_0);
+            A4_0 = rowcol(T2_0, x);
+            A5_0 = rowcol(T2_0, y);
+            A4_1 = rowcol(T2_1, x);
+            A5_1 = rowcol(T2_1, y);
+          }
+          {
+            const ws<R> WJ = weyl_form(J0_2);
+            sp<R> x = slash(WJ, S_E), y = spneg(x);  // J(02) v and J(20) v
+            slash_acc(x, W0, S_2);
+            slash_acc(y, W2, S_0);
+            A2_0 = rowcol(T1_0, x);
+            A3_0 = rowcol(T1_0, y);
+            A2_1 = rowcol(T1_1, x);
+            A3_1 = rowcol(T1_1, y);
+          }
+          {
+            const ws<R> WJ = weyl_form(J1_2);
+            sp<R> x = slash(WJ, S_E), y = spneg(x);  // J(12) v and J(21) v
+            slash_acc(x, W1, S_2);
+            slash_acc(y, W2, S_1);
+            A0_0 = rowcol(T0_0, x);
+            A1_0 = rowcol(T0_0, y);
+            A0_1 = rowcol(T0_1, x);
+            A1_1 = rowcol(T0_1, y);
+          }
+          {
+            const sp<R> z = slash(J0_1, S_2);
+            const cx<R> d0 = rowcol(X.ub[0], z);
+            A0_0 = A0_0 + d0;
+            A2_0 = A2_0 - d0;
+            const cx<R> d1 = rowcol(X.ub[1], z);
+            A0_1 = A0_1 + d1;
+            A2_1 = A2_1 - d1;
+          }
+          {
+            const sp<R> z = slash(J0_2, S_1);
+            const cx<R> d0 = rowcol(X.ub[0], z);
+            A1_0 = A1_0 + d0;
+            A4_0 = A4_0 - d0;
+            const cx<R> d1 = rowcol(X.ub[1], z);
+            A1_1 = A1_1 + d1;
+            A4_1 = A4_1 - d1;
+          }
+          {
+            const sp<R> z = slash(J1_2, S_0);
+            const cx<R> d0 = rowcol(X.ub[0], z);
+            A3_0 = A3_0 + d0;
+            A5_0 = A5_0 - d0;
+            const cx<R> d1 = rowcol(X.ub[1], z);
+            A3_1 = A3_1 + d1;
+            A5_1 = A5_1 - d1;
+          }
+          {
+            const cv<R> V = fcur(X.ub[0], S_E);
+            const cx<R> u = dot(V, J0_1_2), t = dot(V, J0_2_1), m = u + t;
+            A0_0 = A0_0 + u;
+            A5_0 = A5_0 + u;
+            A1_0 = A1_0 + t;
+            A3_0 = A3_0 + t;
+            A2_0 = A2_0 - m;
+            A4_0 = A4_0 - m;
+          }
+          {
+            const cv<R> V = fcur(X.ub[1], S_E);
+            const cx<R> u = dot(V, J0_1_2), t = dot(V, J0_2_1), m = u + t;
+            A0_1 = A0_1 + u;
+            A5_1 = A5_1 + u;
+            A1_1 = A1_1 + t;
+            A3_1 = A3_1 + t;
+            A2_1 = A2_1 - m;
+            A4_1 = A4_1 - m;
+          }
           if constexpr (CM != CM_FMA) {
             const cx<float> Aa0[K] = {A0_0, A1_0, A2_0, A3_0, A4_0, A5_0};
             const cx<float> Aa1[K] = {A0_1, A1_1, A2_1, A3_1, A4_1, A5_1};
@@ -217,5 +218,5 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
 }
 
 // floating-point operations of one full helicity sum (all levels, all loop trips)
-constexpr long FLOPS_HEL_SUM = 28077;
+constexpr long FLOPS_HEL_SUM = 23073;
 }}  // namespace

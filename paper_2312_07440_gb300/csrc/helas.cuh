@@ -132,20 +132,17 @@ struct v4 {
 
 // Colour-ordered 3-gluon vertex and the off-shell gluon propagator,
 // c = -1/K^2 (Feynman gauge, g stripped), K = P1 + P2:
-//   out = c [ -J1 (2P1+P2).J2 + (J1.J2)(P1-P2) + J2 (2P2+P1).J1 ]     (156 flops)
-// vvv returns it, vvv_acc adds it to o (+8 flops).
+//   out = c [ -J1 (2P1+P2).J2 + (J1.J2)(P1-P2) + J2 (2P2+P1).J1 ]     (142 flops)
+// with P1.J1 = P2.J2 = 0 (every current here is conserved), so 2P1.J2 and
+// 2P2.J1 remain.  vvv returns it, vvv_acc adds it to o (+8 flops).
 template <class R, bool ACC>
 __device__ __forceinline__ void vvv_body(cv<R>& o, const cv<R>& J1, const R (&P1)[4], const cv<R>& J2,
                                          const R (&P2)[4], R c) {
-  R a[4], b[4], d[4];
+  R d[4];
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    a[m] = fmadd(R(2), P1[m], P2[m]);
-    b[m] = fmadd(R(2), P2[m], P1[m]);
-    d[m] = P1[m] - P2[m];
-  }
-  const cx<R> s1 = c * dotr(a, J2);
-  const cx<R> s2 = c * dotr(b, J1);
+  for (int m = 0; m < 4; ++m) d[m] = P1[m] - P2[m];
+  const cx<R> s1 = (R(2) * c) * dotr(P1, J2);
+  const cx<R> s2 = (R(2) * c) * dotr(P2, J1);
   const cx<R> s12 = c * dot(J1, J2);
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
@@ -308,6 +305,45 @@ __device__ __forceinline__ sp<R> fprop(const R (&q)[4], R mc, const sp<R>& s) {
             fmadd(mc, s.c[2].i, fmadd(-q2, s.c[1].r, fmadd(q1, s.c[1].i, ap * s.c[0].i)))};
   o.c[3] = {fmadd(mc, s.c[3].r, fmadd(-q2, s.c[0].i, fmadd(q1, s.c[0].r, am * s.c[1].r))),
             fmadd(mc, s.c[3].i, fmadd(q2, s.c[0].r, fmadd(q1, s.c[0].i, am * s.c[1].i)))};
+  return o;
+}
+
+// Row spinor times Jslash: 56 flops from the Weyl-block form
+template <class R>
+__device__ __forceinline__ sp<R> row_slash(const ws<R>& a, const sp<R>& u) {
+  return {{cmac(a.bp, u.c[3], cmul(a.ap, u.c[2])), cmac(a.am, u.c[3], cmul(a.bm, u.c[2])),
+           cmsc(a.bp, u.c[1], cmul(a.am, u.c[0])), cmsc(a.bm, u.c[0], cmul(a.ap, u.c[1]))}};
+}
+
+// Row spinor times the top propagator, u (qc slash + mc)                    (58 flops)
+template <class R>
+__device__ __forceinline__ sp<R> row_prop(const R (&q)[4], R mc, const sp<R>& u) {
+  const R p[4] = {q[0], q[1], -q[2], q[3]};
+  const sp<R> x = fprop(p, mc, sp<R>{{u.c[2], u.c[3], u.c[0], u.c[1]}});
+  return {{x.c[2], x.c[3], x.c[0], x.c[1]}};
+}
+
+// Off-shell current of three gluons in the order a b c from their
+// polarisations and two-gluon currents, c = -1/K^2 of the three; every current
+// is conserved, so only one vertex momentum enters each product   (450 flops)
+template <class R>
+__device__ __forceinline__ cv<R> current3(const cv<R>& A, const cv<R>& B, const cv<R>& C, const cv<R>& AB, const cv<R>& BC,
+                                          const R (&Pa)[4], const R (&Pc)[4], const R (&Pab)[4], const R (&Pbc)[4], R c) {
+  const R c2 = R(2) * c;
+  const cx<R> ga = c * dot(A, BC), gc = c * dot(AB, C);
+  const cx<R> fa = c * dot(B, C) - c2 * dotr(Pa, BC), fc = c * dot(A, B) + c2 * dotr(Pc, AB);
+  const cx<R> fb = (-c2) * dot(A, C), fbc = c2 * dotr(Pbc, A), fab = (-c2) * dotr(Pab, C);
+  cv<R> o;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    cx<R> x = (Pa[m] - Pbc[m]) * ga;
+    x = rmac(Pab[m] - Pc[m], gc, x);
+    x = cmac(A.c[m], fa, x);
+    x = cmac(B.c[m], fb, x);
+    x = cmac(C.c[m], fc, x);
+    x = cmac(AB.c[m], fab, x);
+    o.c[m] = cmac(BC.c[m], fbc, x);
+  }
   return o;
 }
 

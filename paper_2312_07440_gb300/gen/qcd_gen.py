@@ -184,7 +184,8 @@ PAIRS_MAX_K = 6  # colour sums of up to this many orderings by pairs (see emit_p
 ROW_ACCS = 4     # accumulators per top helicity for the row-wise colour sum
 
 FLOPS = {
-    "vvv": 156,      # 3-gluon vertex with folded propagator factor
+    "vvv": 142,      # 3-gluon vertex with folded propagator factor
+    "current3": 450, # three-gluon current from two-gluon ones
     "vvvv_acc": 193, # 4-gluon vertex accumulated
     "slash": 64,     # Jslash psi from the vector J
     "slash_w": 56,   # Jslash psi from J's Weyl-block form
@@ -207,6 +208,60 @@ def mask(seq):
     for x in seq:
         m |= 1 << x
     return m
+
+
+def emit_cut(w, ind, n, em, jref):
+    """Antitop level for three gluons with the fermion line cut after its first
+    gluon: A(abc) = T(a).X(bc) + (ub J(ab)).S(c) + (ub gamma v).J(abc), with
+    X(bc) = J_b S(c) + J(bc) v never propagated, both top helicities."""
+    perms = orderings(n)
+    w(f"{ind}sp<R> S_0;")
+    w(f"{ind}if constexpr (LB < {n}) S_0 = h{n} ? S_0v1 : S_0v0;")
+    w(f"{ind}else S_0 = fprop(Kn.qc[1], Kn.mc[1], slash(W0, S_E));")
+    for g in (1, 2):
+        w(f"{ind}const sp<R> S_{g} = fprop(Kn.qc[{1 << g}], Kn.mc[{1 << g}], slash(W{g}, S_E));")
+    em.count(n, "slash_w", 2)
+    em.count(n, "fprop", 2)
+    k = {p: i for i, p in enumerate(perms)}
+    w(f"{ind}cx<R> {', '.join(f'A{i}_{h}' for i in range(len(perms)) for h in (0, 1))};")
+    for b, c in ((0, 1), (0, 2), (1, 2)):
+        a = 3 - b - c
+        w(f"{ind}{{")
+        w(f"{ind}  const ws<R> WJ = weyl_form({jref((b, c))});")
+        w(f"{ind}  sp<R> x = slash(WJ, S_E), y = spneg(x);  // J({b}{c}) v and J({c}{b}) v")
+        w(f"{ind}  slash_acc(x, W{b}, S_{c});")
+        w(f"{ind}  slash_acc(y, W{c}, S_{b});")
+        for h in (0, 1):
+            w(f"{ind}  A{k[a, b, c]}_{h} = rowcol(T{a}_{h}, x);")
+            w(f"{ind}  A{k[a, c, b]}_{h} = rowcol(T{a}_{h}, y);")
+        em.count(n, "weyl")
+        em.count(n, "slash_w", 3)
+        em.count(n, "sp_add", 2)
+        em.count(n, "rowcol", 4)
+        w(f"{ind}}}")
+    for a, b in ((0, 1), (0, 2), (1, 2)):
+        c = 3 - a - b
+        w(f"{ind}{{")
+        w(f"{ind}  const sp<R> z = slash({jref((a, b))}, S_{c});")
+        for h in (0, 1):
+            w(f"{ind}  const cx<R> d{h} = rowcol(X.ub[{h}], z);")
+            w(f"{ind}  A{k[a, b, c]}_{h} = A{k[a, b, c]}_{h} + d{h};")
+            w(f"{ind}  A{k[b, a, c]}_{h} = A{k[b, a, c]}_{h} - d{h};")
+        em.count(n, "slash")
+        em.count(n, "rowcol", 2)
+        em.count(n, "cadd", 4)
+        w(f"{ind}}}")
+    for h in (0, 1):
+        w(f"{ind}{{")
+        w(f"{ind}  const cv<R> V = fcur(X.ub[{h}], S_E);")
+        w(f"{ind}  const cx<R> u = dot(V, J0_1_2), t = dot(V, J0_2_1), m = u + t;")
+        for p, e in (((0, 1, 2), "+ u"), ((2, 1, 0), "+ u"), ((0, 2, 1), "+ t"), ((1, 2, 0), "+ t"), ((1, 0, 2), "- m"),
+                     ((2, 0, 1), "- m")):
+            w(f"{ind}  A{k[p]}_{h} = A{k[p]}_{h} {e};")
+        em.count(n, "fcur")
+        em.count(n, "dot", 2)
+        em.count(n, "cadd", 7)
+        w(f"{ind}}}")
 
 
 class Emitter:
@@ -251,7 +306,8 @@ def emit_process(name, n, outgoing_gluons, n_identical, hoist_weyl=True, share_f
     w(f"constexpr int NHEL = {2 ** (n + 2)};")
     w(f"constexpr int NDIAG = {diagram_count(n)};")
     w(f"constexpr int MAX_LB = {n};  // helicity levels that can be spread over lanes")
-    njs = sum(math.perm(n, L) // 2 for L in range(3, n + 1))
+    cut = n == 3
+    njs = 0 if cut else sum(math.perm(n, L) // 2 for L in range(3, n + 1))
     w(f"constexpr int NJS = {njs};  // currents of 3+ gluons, one JStore slot each")
     w(f"constexpr int CDEN = {den};")
     w(f"constexpr int IDENT = {n_identical};  // identical outgoing gluons (1/IDENT!)")
@@ -338,6 +394,14 @@ def emit_process(name, n, outgoing_gluons, n_identical, hoist_weyl=True, share_f
         if hoist_weyl:
             w(f"{ind}const ws<R> W{g} = weyl_form(E{g});")
             em.count(g, "weyl")
+        if cut:
+            # the top's side: T(g) = ub Jslash_g prop, the line between gluon g
+            # and the other two
+            m = ((1 << n) - 1) ^ (1 << g)
+            w(f"{ind}const sp<R> T{g}_0 = row_prop(Kn.qc[{m}], Kn.mc[{m}], row_slash(W{g}, X.ub[0]));")
+            w(f"{ind}const sp<R> T{g}_1 = row_prop(Kn.qc[{m}], Kn.mc[{m}], row_slash(W{g}, X.ub[1]));")
+            em.count(g, "slash_w", 2)
+            em.count(g, "fprop", 2)
         if g == 0 and hoist_weyl:
             # S(0) depends on the antitop helicity and on gluon 0's, which is
             # fixed: both antitop variants are formed here once instead of at
@@ -364,6 +428,16 @@ def emit_process(name, n, outgoing_gluons, n_identical, hoist_weyl=True, share_f
                         alias[sq] = expr
                     else:
                         w(f"{ind}const cv<R> {nm} = {expr};")
+                    continue
+                if cut and L == 3:
+                    # (1, 0, 2) is minus the sum of the two orders with gluon 0 first
+                    if sq[0] == 0:
+                        canon[sq] = nm
+                        a, b, c = sq
+                        w(f"{ind}const cv<R> {nm} = current3({jref((a,))}, {jref((b,))}, {jref((c,))}, {jref((a, b))}, "
+                          f"{jref((b, c))}, Kn.P[{1 << a}], Kn.P[{1 << c}], Kn.P[{mask((a, b))}], Kn.P[{mask((b, c))}], "
+                          f"Kn.cg[7]);")
+                        em.count(g, "current3")
                     continue
                 canon[sq] = nm
                 m = mask(sq)
@@ -438,7 +512,10 @@ def emit_process(name, n, outgoing_gluons, n_identical, hoist_weyl=True, share_f
             ops.append(("line", f"const sp<R> {nm} = fprop(Kn.qc[{mask(rho)}], Kn.mc[{mask(rho)}], t{nm});"))
             em.count(n, "fprop")
             visit(rho)
-    visit(())
+    if cut:
+        emit_cut(w, ind, n, em, jref)
+    else:
+        visit(())
 
     def share_key(a, b):
         ca = a if a in canon else tuple(reversed(a))
@@ -452,7 +529,8 @@ def emit_process(name, n, outgoing_gluons, n_identical, hoist_weyl=True, share_f
                 uses.setdefault(share_key(a, b)[0], []).append(i)
     assert all(len(u) == 2 for u in uses.values())
     share_gaps = sorted(u[1] - u[0] for u in uses.values())
-    w(f"{ind}constexpr bool SH = sizeof(R) == 8;  // share every repeated slash (FP64)")
+    if not cut:
+        w(f"{ind}constexpr bool SH = sizeof(R) == 8;  // share every repeated slash (FP64)")
     for i, op in enumerate(ops):
         if op[0] == "line":
             w(f"{ind}{op[1]}")
