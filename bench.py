@@ -110,7 +110,7 @@ def source_sha(process, mode):
     the launch code and every header except other processes' generated
     amplitude code and the surrogate network's tensor-core kernels (the
     host-only event-file I/O holds no device code)."""
-    mlp_only = ("gemm_tc.cuh", "mlp_infer_tc.cuh")
+    mlp_only = ("gemm_tc.cuh", "mlp_infer_tc.cuh", "wgrad_tc.cuh")
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2312_07440_gb300", "csrc")
     tu = f"proc_{process}_{'mixed' if mode.startswith('mixed') else mode}.cu"
