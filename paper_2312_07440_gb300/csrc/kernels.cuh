@@ -235,6 +235,17 @@ __device__ __forceinline__ void reduce_sums(const RwArgs& a, const double2* sacc
   }
 }
 
+// Proc::Common (optional): what the evaluations of one event have in common
+// where a point changes couplings only and never the momenta
+template <class P, class R, int LB, class = void>
+struct Shared : std::false_type {
+  struct type {};
+};
+template <class P, class R, int LB>
+struct Shared<P, R, LB, std::void_t<typename P::template Common<R, LB>>> : std::true_type {
+  using type = typename P::template Common<R, LB>;
+};
+
 // MINB: resident blocks of 256 threads per SM the register allocation must
 // allow (1: up to 255 registers; 2: 128, for small processes whose FP32
 // kernels are latency-bound at 8 warps per SM).
@@ -281,6 +292,8 @@ __global__ void __launch_bounds__(256, MINB) k_reweight(const __grid_constant__ 
     for (int i = 0; i < NEXT; ++i)
 #pragma unroll
       for (int m = 0; m < 4; ++m) load_mom(p[i][m], __ldg(a.mom + ((long long)(i * 4 + m)) * a.ld + evc));
+    typename Shared<Proc, R, LB>::type common;
+    if constexpr (Shared<Proc, R, LB>::value) Proc::template common<R, LB>(p, lane, gmask, common);
     // One call site for every evaluation (original, then each point), so that
     // identical parameters give bitwise identical |M|^2 and r == 1 exactly.
     // Points that differ in the overall coupling only share an evaluation
@@ -300,7 +313,12 @@ __global__ void __launch_bounds__(256, MINB) k_reweight(const __grid_constant__ 
       // g g -> t tbar g wait for instructions as often as they issue: 131,072
       // events x 64 points 10.24 -> 9.28 ms; every fourth evaluation: 9.58 ms)
       if constexpr (sizeof(R) == 4) __syncthreads();
-      const double s = eval_point<Proc, R, LB>(p, a.pt[a.me_only ? 0 : a.kin_rep[k]], lane, gmask);
+      const PointDev& pk = a.pt[a.me_only ? 0 : a.kin_rep[k]];
+      double s;
+      if constexpr (Shared<Proc, R, LB>::value)
+        s = Proc::template point<R, LB>(common, pk, lane, gmask);
+      else
+        s = eval_point<Proc, R, LB>(p, pk, lane, gmask);
       if (a.me_only) {
         if (leader) a.me0[ev] = s * a.pt[0].cscale;
         break;
