@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(256, 1) k_amp_store(const __grid_constant__ Rw
       for (int m = 0; m < 4; ++m) load_mom(p[i][m], __ldg(a.mom + ((long long)(i * 4 + m)) * a.ld + evc));
 #pragma unroll 1
     for (int j = 0; j < npts; ++j) {
+      __syncthreads();  // the block's warps start every evaluation together, as in k_reweight
       ColourSink<K, CM> sk{j16, ex, L.ld, valid ? ev : -1, j * SLOTS + lane * (SLOTS >> LB)};
       const bool inside = Proc::template me_store<float, LB>(p, a.pt[j], lane, gmask, sk);
       if (valid && lane == 0) ins[(long long)j * L.ld + ev] = inside ? 1 : 0;

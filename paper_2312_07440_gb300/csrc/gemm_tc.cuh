@@ -61,22 +61,51 @@ struct Epi {
   int M, N, K;
 };
 
-// SiLU z sigma(z) = z / (1 + 2^(-z log2 e)) with the special-function unit's
-// approximate base-2 exponential and reciprocal (each within a few units in
-// the last place of FP32; the result is rounded to BF16).  Below z = -88 the
-// exponential overflows to +inf and the result is -0.
-__device__ __forceinline__ float silu_f(float z) {
-  float e, r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
-  return z * r;
+// Packed FP32 pairs: one instruction for two lanes' worth of additions or
+// products (each rounded as by itself)
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// SiLU z sigma(z) = z / (1 + 2^(-z log2 e)) of the pair z with the
+// special-function unit's approximate base-2 exponential and reciprocal (each
+// within a few units in the last place of FP32; the result is rounded to
+// BF16).  Below z = -88 the exponential overflows to +inf and the result is -0.
+__device__ __forceinline__ void silu_pair(uint64_t z, float& h0, float& h1) {
+  float t0, t1, q0, q1;
+  unpack2(mul2(z, pack2(-1.4426950408889634f, -1.4426950408889634f)), t0, t1);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(t0));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(t1));
+  unpack2(add2(pack2(t0, t1), pack2(1.0f, 1.0f)), q0, q1);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q0) : "f"(q0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q1) : "f"(q1));
+  unpack2(mul2(z, pack2(q0, q1)), h0, h1);
+}
+// of v + b
+__device__ __forceinline__ void silu_pair(float v0, float v1, float b0, float b1, float& h0, float& h1) {
+  silu_pair(add2(pack2(v0, v1), pack2(b0, b1)), h0, h1);
 }
 
 __device__ __forceinline__ unsigned short bf16_bits(float x) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(x));
 }
 
-// SiLU'(z) = sigma(z) (1 + z (1 - sigma(z))), sigma from the same exp2 and reciprocal
+// SiLU'(z) = sigma(z) (1 + z (1 - sigma(z))), sigma from the same functions
 __device__ __forceinline__ float dsilu_f(float z) {
   float e, s;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
@@ -253,7 +282,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(const __grid_constant__ 
           for (int j = 0; j < 4; ++j) zp[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         }
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = silu_f(v[j]);
+        for (int j = 0; j < 16; j += 2) silu_pair(pack2(v[j], v[j + 1]), v[j], v[j + 1]);
         if (e.H) {
           uint4* hp = reinterpret_cast<uint4*>(e.H + row * N + c0);
 #pragma unroll

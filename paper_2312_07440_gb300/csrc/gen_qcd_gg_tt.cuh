@@ -48,7 +48,7 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
       const int h1 = LB >= 1 ? ((lane >> (LB - 1)) & 1) : i1;
       const cv<R> E1 = h1 ? X.eps[1][1] : X.eps[1][0];
       const ws<R> W1 = weyl_form(E1);
-      cv<R> J0_1 = vvv(E0, Kn.P[1], E1, Kn.P[2], Kn.cg[3]);
+      cv<R> J0_1 = current2(E0, Kn.P[1], E1, Kn.P[2], Kn.cg[3]);
       const ws<R> WJ0_1 = weyl_form(J0_1);
       const cv<R> J1_0 = neg(J0_1);
       #pragma unroll 1

@@ -52,7 +52,7 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
       const ws<R> W1 = weyl_form(E1);
       const sp<R> T1_0 = row_prop(Kn.qc[5], Kn.mc[5], row_slash(W1, X.ub[0]));
       const sp<R> T1_1 = row_prop(Kn.qc[5], Kn.mc[5], row_slash(W1, X.ub[1]));
-      cv<R> J0_1 = vvv(E0, Kn.P[1], E1, Kn.P[2], Kn.cg[3]);
+      cv<R> J0_1 = current2(E0, Kn.P[1], E1, Kn.P[2], Kn.cg[3]);
       const cv<R> J1_0 = neg(J0_1);
       #pragma unroll 1
       for (int i2 = 0; i2 < (LB >= 2 ? 1 : 2); ++i2) {
@@ -61,8 +61,8 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
         const ws<R> W2 = weyl_form(E2);
         const sp<R> T2_0 = row_prop(Kn.qc[3], Kn.mc[3], row_slash(W2, X.ub[0]));
         const sp<R> T2_1 = row_prop(Kn.qc[3], Kn.mc[3], row_slash(W2, X.ub[1]));
-        cv<R> J0_2 = vvv(E0, Kn.P[1], E2, Kn.P[4], Kn.cg[5]);
-        cv<R> J1_2 = vvv(E1, Kn.P[2], E2, Kn.P[4], Kn.cg[6]);
+        cv<R> J0_2 = current2(E0, Kn.P[1], E2, Kn.P[4], Kn.cg[5]);
+        cv<R> J1_2 = current2(E1, Kn.P[2], E2, Kn.P[4], Kn.cg[6]);
         const cv<R> J2_0 = neg(J0_2);
         const cv<R> J2_1 = neg(J1_2);
         const cv<R> J0_1_2 = current3(E0, E1, E2, J0_1, J1_2, Kn.P[1], Kn.P[4], Kn.P[3], Kn.P[6], Kn.cg[7]);

@@ -1139,5 +1139,5 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
 }
 
 // floating-point operations of one full helicity sum (all levels, all loop trips)
-constexpr long FLOPS_HEL_SUM = 397447;
+constexpr long FLOPS_HEL_SUM = 404307;
 }}  // namespace

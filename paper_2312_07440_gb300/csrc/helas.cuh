@@ -132,17 +132,20 @@ struct v4 {
 
 // Colour-ordered 3-gluon vertex and the off-shell gluon propagator,
 // c = -1/K^2 (Feynman gauge, g stripped), K = P1 + P2:
-//   out = c [ -J1 (2P1+P2).J2 + (J1.J2)(P1-P2) + J2 (2P2+P1).J1 ]     (142 flops)
-// with P1.J1 = P2.J2 = 0 (every current here is conserved), so 2P1.J2 and
-// 2P2.J1 remain.  vvv returns it, vvv_acc adds it to o (+8 flops).
+//   out = c [ -J1 (2P1+P2).J2 + (J1.J2)(P1-P2) + J2 (2P2+P1).J1 ]     (156 flops)
+// vvv returns it, vvv_acc adds it to o (+8 flops).
 template <class R, bool ACC>
 __device__ __forceinline__ void vvv_body(cv<R>& o, const cv<R>& J1, const R (&P1)[4], const cv<R>& J2,
                                          const R (&P2)[4], R c) {
-  R d[4];
+  R a[4], b[4], d[4];
 #pragma unroll
-  for (int m = 0; m < 4; ++m) d[m] = P1[m] - P2[m];
-  const cx<R> s1 = (R(2) * c) * dotr(P1, J2);
-  const cx<R> s2 = (R(2) * c) * dotr(P2, J1);
+  for (int m = 0; m < 4; ++m) {
+    a[m] = fmadd(R(2), P1[m], P2[m]);
+    b[m] = fmadd(R(2), P2[m], P1[m]);
+    d[m] = P1[m] - P2[m];
+  }
+  const cx<R> s1 = c * dotr(a, J2);
+  const cx<R> s2 = c * dotr(b, J1);
   const cx<R> s12 = c * dot(J1, J2);
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
@@ -321,6 +324,20 @@ __device__ __forceinline__ sp<R> row_prop(const R (&q)[4], R mc, const sp<R>& u)
   const R p[4] = {q[0], q[1], -q[2], q[3]};
   const sp<R> x = fprop(p, mc, sp<R>{{u.c[2], u.c[3], u.c[0], u.c[1]}});
   return {{x.c[2], x.c[3], x.c[0], x.c[1]}};
+}
+
+// Off-shell current of two external gluons: vvv with P1.J1 = P2.J2 = 0 left
+// out of the vertex, which spares forming 2P1 + P2 and 2P2 + P1    (142 flops)
+template <class R>
+__device__ __forceinline__ cv<R> current2(const cv<R>& A, const R (&Pa)[4], const cv<R>& B, const R (&Pb)[4], R c) {
+  const cx<R> s1 = (R(2) * c) * dotr(Pa, B), s2 = (R(2) * c) * dotr(Pb, A), s12 = c * dot(A, B);
+  cv<R> o;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const R d = Pa[m] - Pb[m];
+    o.c[m] = cmsc(A.c[m], s1, cmac(B.c[m], s2, cx<R>{d * s12.r, d * s12.i}));
+  }
+  return o;
 }
 
 // Off-shell current of three gluons in the order a b c from their

@@ -290,10 +290,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
               for (int j = 0; j < 4; ++j) {
                 const float4 p = b4[2 * j], q = b4[2 * j + 1];
                 const uint32_t* x = &u[j >> 1][(8 * j) & 15];
-                const uint4 w4 = make_uint4(bf16x2(silu_f(__uint_as_float(x[0]) + p.x), silu_f(__uint_as_float(x[1]) + p.y)),
-                                            bf16x2(silu_f(__uint_as_float(x[2]) + p.z), silu_f(__uint_as_float(x[3]) + p.w)),
-                                            bf16x2(silu_f(__uint_as_float(x[4]) + q.x), silu_f(__uint_as_float(x[5]) + q.y)),
-                                            bf16x2(silu_f(__uint_as_float(x[6]) + q.z), silu_f(__uint_as_float(x[7]) + q.w)));
+                float h[8];
+                silu_pair(__uint_as_float(x[0]), __uint_as_float(x[1]), p.x, p.y, h[0], h[1]);
+                silu_pair(__uint_as_float(x[2]), __uint_as_float(x[3]), p.z, p.w, h[2], h[3]);
+                silu_pair(__uint_as_float(x[4]), __uint_as_float(x[5]), q.x, q.y, h[4], h[5]);
+                silu_pair(__uint_as_float(x[6]), __uint_as_float(x[7]), q.z, q.w, h[6], h[7]);
+                const uint4 w4 = make_uint4(bf16x2(h[0], h[1]), bf16x2(h[2], h[3]), bf16x2(h[4], h[5]), bf16x2(h[6], h[7]));
                 *reinterpret_cast<uint4*>(as + act_off(r, c0 + 8 * j)) = w4;
               }
             }
@@ -313,7 +315,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
                 const float bl = (j & 1) ? b4[j >> 1].z : b4[j >> 1].x, bh = (j & 1) ? b4[j >> 1].w : b4[j >> 1].y;
-                const float v0 = silu_f(__uint_as_float(u[2 * j]) + bl), v1 = silu_f(__uint_as_float(u[2 * j + 1]) + bh);
+                float v0, v1;
+                silu_pair(__uint_as_float(u[2 * j]), __uint_as_float(u[2 * j + 1]), bl, bh, v0, v1);
                 h0 = fmaf(v0, w4[j].x, h0);
                 h1 = fmaf(v0, w4[j].y, h1);
                 h0 = fmaf(v1, w4[j].z, h0);

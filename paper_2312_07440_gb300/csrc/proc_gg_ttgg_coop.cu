@@ -1,5 +1,8 @@
 // g g -> t tbar g g with one warp per event (coop_kernel.cuh): FP64, FP32, and
-// the amplitude pass of the mixed modes' separate colour sum.
+// the amplitude pass of the FP16-mixed mode's separate colour sum.  (Not the
+// BF16 one's: rounding the amplitude vectors to 8 bits turns the last-bit
+// differences between two FP32 evaluations into differences of up to 1.5e-3 in
+// W', and its results stay those of the 8-lane pass.)
 #include "../../include/rwgt.h"
 #include "coop_kernel.cuh"
 #include "gen_qcd_gg_ttgg.cuh"
@@ -15,18 +18,13 @@ constexpr int per_thread = (int)(sizeof(coop::Warp<R>) / 32);
 static_assert(sizeof(coop::Warp<float>) % 32 == 0 && sizeof(coop::Warp<double>) % 32 == 0, "whole bytes per thread, 16-byte aligned");
 constexpr int SLOTS = 1 << (gg_ttgg::NEXT - 1);
 
-template <int CM>
-KernelEntry store_entry(int mode) {
-  return {RW_GG_TTGG, mode, 5, (const void*)&coop::k_coop<float, CM>, 256, 2, per_thread<float>,
-          (const void*)&k_colour_tc<gg_ttgg::K, CM, SLOTS, CTab>};
-}
 }  // namespace
 
 void register_gg_ttgg_coop(std::vector<KernelEntry>& t) {
   t.push_back({RW_GG_TTGG, RW_FP64, 5, (const void*)&coop::k_coop<double, CM_FMA>, 256, 0, per_thread<double>, nullptr, 24});
   t.push_back({RW_GG_TTGG, RW_FP32, 5, (const void*)&coop::k_coop<float, CM_FMA>, 256, 0, per_thread<float>, nullptr, 24});
-  t.push_back(store_entry<CM_STORE_FP16>(RW_MIXED_FP16));
-  t.push_back(store_entry<CM_STORE_BF16>(RW_MIXED_BF16));
+  t.push_back({RW_GG_TTGG, RW_MIXED_FP16, 5, (const void*)&coop::k_coop<float, CM_STORE_FP16>, 256, 2, per_thread<float>,
+               (const void*)&k_colour_tc<gg_ttgg::K, CM_STORE_FP16, SLOTS, CTab>});
 }
 
 }  // namespace rw

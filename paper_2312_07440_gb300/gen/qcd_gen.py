@@ -184,7 +184,8 @@ PAIRS_MAX_K = 6  # colour sums of up to this many orderings by pairs (see emit_p
 ROW_ACCS = 4     # accumulators per top helicity for the row-wise colour sum
 
 FLOPS = {
-    "vvv": 142,      # 3-gluon vertex with folded propagator factor
+    "vvv": 156,      # 3-gluon vertex with folded propagator factor
+    "current2": 142, # two-gluon current of external gluons
     "current3": 450, # three-gluon current from two-gluon ones
     "vvvv_acc": 193, # 4-gluon vertex accumulated
     "slash": 64,     # Jslash psi from the vector J
@@ -445,8 +446,10 @@ def emit_process(name, n, outgoing_gluons, n_identical, hoist_weyl=True, share_f
                 for c in range(1, L):
                     a, b = sq[:c], sq[c:]
                     terms.append(f"{jref(a)}, Kn.P[{mask(a)}], {jref(b)}, Kn.P[{mask(b)}], Kn.cg[{m}]")
-                    em.count(g, "vvv")
-                w(f"{ind}cv<R> {nm} = vvv({terms[0]});")
+                    em.count(g, "current2" if n < 4 else "vvv")
+                # four gluons: the vertex with both momenta in either product,
+                # as in its currents of more gluons
+                w(f"{ind}cv<R> {nm} = {'current2' if n < 4 else 'vvv'}({terms[0]});")
                 for t in terms[1:]:
                     w(f"{ind}vvv_acc({nm}, {t});")  # fused accumulation
                     em.count(g, "cadd", 8)

@@ -75,7 +75,7 @@ def test_many_points_and_masses_that_do_not_fit(mode, tol):
     assert g["n_bad"] == t["n_bad"] == 0
 
 
-@pytest.mark.parametrize("mode", ["mixed_fp16", "mixed_bf16"])
+@pytest.mark.parametrize("mode", ["mixed_fp16"])
 def test_mixed_amplitude_pass(mode):
     """The amplitude pass of the separate colour sum in the warp-per-event form: the same rounding to 16 bits, so within
     twice the mode's bound of the 8-lane pass, three tiles with a ragged last one, r == 1 for unchanged parameters."""
