@@ -268,55 +268,65 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
           const bool next = Pn < pairs && 2 * Pn + s < tiles;  // a next tile for this slot
           unsigned char* as = act + (size_t)s * ACT_BYTES;
           if (last && next) load_features(a, (2 * Pn + s) * BM + r, cq, fs);  // in flight during the head
+          // 16 columns at a time, the next 16 in flight (tensor memory, bias)
+          // while these are computed; the first bias before the wait
+          uint32_t u[2][16];
+          float4 b4[2][4];
+          auto load_bias = [&](int ch) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              b4[ch & 1][j] = __ldg(reinterpret_cast<const float4*>(bias + cq * 64 + ch * 16) + j);
+          };
+          load_bias(0);
           if (!(ok = mbar_wait(b_full + 8 * s, (full_ph >> s) & 1u, a.err, 14, abort))) break;
           full_ph ^= 1u << s;
           tc_fence_after();
           const uint32_t tacc = tmem + (uint32_t)(s * N) + lane_base;
           float h0 = 0.0f, h1 = 0.0f;
+          tmem_ld16_nw(tacc + (uint32_t)(cq * 64), u[0]);
           if (!last) {
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              // 32 columns; the bias loads are in flight with the tensor-memory loads
-              const int c0 = cq * 64 + half * 32;
-              uint32_t u[2][16];
-              tmem_ld16_nw(tacc + (uint32_t)c0, u[0]);
-              tmem_ld16_nw(tacc + (uint32_t)(c0 + 16), u[1]);
-              float4 b4[8];
+            for (int ch = 0; ch < 4; ++ch) {
+              const int c0 = cq * 64 + ch * 16;
+              tmem_wait_ld16(u[ch & 1]);
+              if (ch < 3) {
+                tmem_ld16_nw(tacc + (uint32_t)(c0 + 16), u[(ch + 1) & 1]);
+                load_bias(ch + 1);
+              }
+              // the next layer's A operand: 16 columns = two 16-byte chunks
 #pragma unroll
-              for (int j = 0; j < 8; ++j) b4[j] = __ldg(reinterpret_cast<const float4*>(bias + c0) + j);
-              tmem_wait_ld();
-              // the next layer's A operand: 32 columns = four 16-byte chunks
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const float4 p = b4[2 * j], q = b4[2 * j + 1];
-                const uint32_t* x = &u[j >> 1][(8 * j) & 15];
+              for (int j = 0; j < 2; ++j) {
+                const float4 p = b4[ch & 1][2 * j], q = b4[ch & 1][2 * j + 1];
+                const uint32_t* x = &u[ch & 1][8 * j];
                 float h[8];
                 silu_pair(__uint_as_float(x[0]), __uint_as_float(x[1]), p.x, p.y, h[0], h[1]);
                 silu_pair(__uint_as_float(x[2]), __uint_as_float(x[3]), p.z, p.w, h[2], h[3]);
                 silu_pair(__uint_as_float(x[4]), __uint_as_float(x[5]), q.x, q.y, h[4], h[5]);
                 silu_pair(__uint_as_float(x[6]), __uint_as_float(x[7]), q.z, q.w, h[6], h[7]);
-                const uint4 w4 = make_uint4(bf16x2(h[0], h[1]), bf16x2(h[2], h[3]), bf16x2(h[4], h[5]), bf16x2(h[6], h[7]));
-                *reinterpret_cast<uint4*>(as + act_off(r, c0 + 8 * j)) = w4;
+                *reinterpret_cast<uint4*>(as + act_off(r, c0 + 8 * j)) =
+                    make_uint4(bf16x2(h[0], h[1]), bf16x2(h[2], h[3]), bf16x2(h[4], h[5]), bf16x2(h[6], h[7]));
               }
             }
           } else {
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) {
-              // 16 columns with their bias and output weights ([c][2]: two columns per float4)
+              // with their output weights ([c][2]: two columns per float4)
               const int c0 = cq * 64 + ch * 16;
-              uint32_t u[16];
-              tmem_ld16_nw(tacc + (uint32_t)c0, u);
-              float4 b4[4], w4[8];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) b4[j] = __ldg(reinterpret_cast<const float4*>(bias + c0) + j);
+              float4 w4[8];
 #pragma unroll
               for (int j = 0; j < 8; ++j) w4[j] = __ldg(reinterpret_cast<const float4*>(a.w_out + 2 * c0) + j);
-              tmem_wait_ld();
+              tmem_wait_ld16(u[ch & 1]);
+              if (ch < 3) {
+                tmem_ld16_nw(tacc + (uint32_t)(c0 + 16), u[(ch + 1) & 1]);
+                load_bias(ch + 1);
+              }
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
-                const float bl = (j & 1) ? b4[j >> 1].z : b4[j >> 1].x, bh = (j & 1) ? b4[j >> 1].w : b4[j >> 1].y;
+                const float4 p = b4[ch & 1][j >> 1];
+                const float bl = (j & 1) ? p.z : p.x, bh = (j & 1) ? p.w : p.y;
+                const uint32_t* x = &u[ch & 1][2 * j];
                 float v0, v1;
-                silu_pair(__uint_as_float(u[2 * j]), __uint_as_float(u[2 * j + 1]), bl, bh, v0, v1);
+                silu_pair(__uint_as_float(x[0]), __uint_as_float(x[1]), bl, bh, v0, v1);
                 h0 = fmaf(v0, w4[j].x, h0);
                 h1 = fmaf(v0, w4[j].y, h1);
                 h0 = fmaf(v1, w4[j].z, h0);
