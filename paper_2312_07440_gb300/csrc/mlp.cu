@@ -611,7 +611,7 @@ int launch_mlp_infer(rw_mlp* m, const float* x, long long n, float* out) {
   a.L = L;
   const long long pairs = ((n + tcg::BM - 1) / tcg::BM + 1) / 2;
   const int grid = (int)std::max(1LL, std::min<long long>(pairs, m->sm_count));
-  tcg::k_mlp_infer<<<grid, tcg::THREADS, tcg::inf::SMEM_BYTES, m->stream>>>(tw, a);
+  tcg::k_mlp_infer<<<grid, tcg::inf::THREADS, tcg::inf::SMEM_BYTES, m->stream>>>(tw, a);
   return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "inference kernel launch");
 }
 

@@ -28,10 +28,14 @@
 //              its ring slot and each layer to the slot's "full" barrier;
 //   warps 2-17 the epilogue, four per lane quarter and one 64-column quarter
 //              (one k-block of the next layer's A operand) each; they also
-//              write the split features of each new tile into its slot, and
 //              compute the output layer (the column quarters' partial sums
 //              meet in the slot's free activation k-blocks; the last warp to
-//              arrive adds them in a fixed order).
+//              arrive adds them in a fixed order);
+//   warps 18-19 the split features of each new tile: loaded while the previous
+//              tile is computed, written into its slot as soon as that tile's
+//              last MMAs have read it, beside the output layer (written by the
+//              epilogue warps after it, they doubled that layer's epilogue,
+//              3.2k -> 7k cycles).
 // Every wait is bounded (~2^31 cycles): on a timeout the error flag is set,
 // every role stops, the MMA thread drains its MMAs, the TMA thread waits for
 // its loads in flight, and the tensor memory is freed before the kernel
@@ -46,6 +50,8 @@ constexpr int N = 256;                               // hidden width
 constexpr int WSTAGES = 3;                           // weight ring depth
 constexpr int MAX_LAYERS = 8;                        // input layer + hidden layers
 constexpr int MAX_IN = 40;                           // 3 n_in <= 128: the split input fits two k-blocks
+constexpr int FEATURE_WARP = 2 + EPI_WARPS;          // the first of two
+constexpr int THREADS = 32 * (FEATURE_WARP + 2);
 constexpr int KB_HIDDEN = N / BK;                    // k-blocks of a hidden layer
 constexpr size_t KB_BYTES = (size_t)BM * 128;        // one k-block of a tile's activations (16 KB)
 constexpr size_t ACT_BYTES = KB_HIDDEN * KB_BYTES;   // a tile's activations (64 KB)
@@ -63,7 +69,7 @@ struct InferArgs {
   float* out;                           // [M][2]
   int* err;                             // set to a nonzero code when a wait gives up
   long long M;
-  int n_in;                             // even, <= MAX_IN
+  int n_in;                             // a multiple of 8, <= MAX_IN
   int kb0;                              // k-blocks of the split input layer: ceil(3 n_in / 64)
   int L;                                // layers before the output layer (input + hidden)
 };
@@ -77,44 +83,51 @@ __device__ __forceinline__ uint32_t act_off(int r, int c) {
   return (uint32_t)((c >> 6) * inf::KB_BYTES + r * 128 + ((((w >> 3) ^ r) & 7) << 4) + ((w & 7) << 1));
 }
 
-// the split features of one row (this thread's share of the feature pairs)
-struct FeatureShare {
-  float v[2 * 5];  // up to 5 pairs: ceil(MAX_IN / 2 / 4)
+// the features of one row, as quadruples
+struct Features {
+  float4 v[inf::MAX_IN / 4];
 };
 
-__device__ __forceinline__ void load_features(const InferArgs& a, long long row, int cq, FeatureShare& f) {
-  const int pairs = a.n_in >> 1, per = (pairs + 3) >> 2, p0 = cq * per;
+__device__ __forceinline__ void load_features(const InferArgs& a, long long row, bool aligned, Features& f) {
   const bool live = row < a.M;
   const float* xr = a.x + (live ? row : 0) * a.n_in;
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int p = p0 + i;
-    const bool ok = live && i < per && p < pairs;
-    f.v[2 * i] = ok ? __ldg(xr + 2 * p) : 0.0f;
-    f.v[2 * i + 1] = ok ? __ldg(xr + 2 * p + 1) : 0.0f;
+  for (int i = 0; i < inf::MAX_IN / 4; ++i) {
+    if (!live || 4 * i >= a.n_in)
+      f.v[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    else if (aligned)
+      f.v[i] = __ldg(reinterpret_cast<const float4*>(xr) + i);
+    else
+      f.v[i] = make_float4(__ldg(xr + 4 * i), __ldg(xr + 4 * i + 1), __ldg(xr + 4 * i + 2), __ldg(xr + 4 * i + 3));
   }
 }
 
-// columns [0, n) x_h, [n, 2n) x_l, [2n, 3n) x_h, [3n, 64 kb0) zero
-__device__ __forceinline__ void store_features(unsigned char* act, const InferArgs& a, int r, int cq,
-                                               const FeatureShare& f) {
-  const int n = a.n_in, pairs = n >> 1, per = (pairs + 3) >> 2, p0 = cq * per;
+// columns [0, n) x_h, [n, 2n) x_l, [2n, 3n) x_h, [3n, 64 kb0) zero, in
+// 16-byte chunks of 8 columns
+__device__ __forceinline__ void store_features(unsigned char* act, const InferArgs& a, int r, const Features& f) {
+  const int n = a.n_in;
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int p = p0 + i;
-    if (i >= per || p >= pairs) break;
-    const float x0 = f.v[2 * i], x1 = f.v[2 * i + 1];
-    const float h0 = __bfloat162float(__float2bfloat16_rn(x0)), h1 = __bfloat162float(__float2bfloat16_rn(x1));
-    const uint32_t hi = bf16x2(h0, h1), lo = bf16x2(x0 - h0, x1 - h1);
-    *reinterpret_cast<uint32_t*>(act + act_off(r, 2 * p)) = hi;
-    *reinterpret_cast<uint32_t*>(act + act_off(r, n + 2 * p)) = lo;
-    *reinterpret_cast<uint32_t*>(act + act_off(r, 2 * n + 2 * p)) = hi;
+  for (int i = 0; i < inf::MAX_IN / 8; ++i) {
+    if (8 * i >= n) break;
+    const float x[8] = {f.v[2 * i].x,     f.v[2 * i].y,     f.v[2 * i].z,     f.v[2 * i].w,
+                        f.v[2 * i + 1].x, f.v[2 * i + 1].y, f.v[2 * i + 1].z, f.v[2 * i + 1].w};
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float h0 = __bfloat162float(__float2bfloat16_rn(x[2 * j])), h1 = __bfloat162float(__float2bfloat16_rn(x[2 * j + 1]));
+      hi[j] = bf16x2(h0, h1);
+      lo[j] = bf16x2(x[2 * j] - h0, x[2 * j + 1] - h1);
+    }
+    const uint4 h = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(act + act_off(r, 8 * i)) = h;
+    *reinterpret_cast<uint4*>(act + act_off(r, n + 8 * i)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    *reinterpret_cast<uint4*>(act + act_off(r, 2 * n + 8 * i)) = h;
   }
-  if (cq == 3)
-    for (int c = 3 * n; c < 64 * a.kb0; c += 2) *reinterpret_cast<uint32_t*>(act + act_off(r, c)) = 0u;
+  for (int c = 3 * n; c < 64 * a.kb0; c += 8)
+    *reinterpret_cast<uint4*>(act + act_off(r, c)) = make_uint4(0u, 0u, 0u, 0u);
 }
 
-__global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant__ CUtensorMap tmW, const InferArgs a) {
+__global__ void __launch_bounds__(inf::THREADS, 1) k_mlp_infer(const __grid_constant__ CUtensorMap tmW, const InferArgs a) {
   using namespace inf;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base =
@@ -122,11 +135,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
   unsigned char* act = base;                      // [2 slots][4 k-blocks][128 rows][128 B]
   unsigned char* wring = base + 2 * ACT_BYTES;    // [WSTAGES][256 rows][128 B]
   uint64_t* bars = reinterpret_cast<uint64_t*>(wring + WSTAGES * WBOX_BYTES);
-  // barrier slots: wfull[WSTAGES], wempty[WSTAGES], ready[2], full[2], drain
+  // barrier slots: wfull[WSTAGES], wempty[WSTAGES], ready[2], full[2], drain, features[2],
+  // free[2] (the slot's tile has been read by its last MMAs)
   const uint32_t b_wfull = smem_u32(bars), b_wempty = smem_u32(bars + WSTAGES);
   const uint32_t b_ready = smem_u32(bars + 2 * WSTAGES), b_full = smem_u32(bars + 2 * WSTAGES + 2);
   const uint32_t b_drain = smem_u32(bars + 2 * WSTAGES + 4);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * WSTAGES + 5);
+  const uint32_t b_feat = smem_u32(bars + 2 * WSTAGES + 5);
+  const uint32_t b_free = smem_u32(bars + 2 * WSTAGES + 7);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * WSTAGES + 9);
   __shared__ int abort_flag;
   __shared__ int head_count[8];  // [slot][lane quarter]: column quarters done
 
@@ -144,6 +160,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
     for (int s = 0; s < 2; ++s) {
       mbar_init(b_ready + 8 * s, EPI_WARPS);  // one arrival per epilogue warp
       mbar_init(b_full + 8 * s, 1);
+      mbar_init(b_feat + 8 * s, 2);
+      mbar_init(b_free + 8 * s, 1);
     }
     mbar_init(b_drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -201,7 +219,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16(BM, N);
       int stage = 0;
-      uint32_t phase = 0, ready_ph = 0;  // bit s: the parity slot s waits for next
+      uint32_t phase = 0, ready_ph = 0, feat_ph = 0;  // bit s: the parity slot s waits for next
       bool ok = true;
       for (long long P = blockIdx.x; ok && P < pairs; P += gridDim.x) {
         const int ns = 2 * P + 1 < tiles ? 2 : 1;
@@ -210,6 +228,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
           for (int s = 0; ok && s < ns; ++s) {
             if (!(ok = mbar_wait(b_ready + 8 * s, (ready_ph >> s) & 1u, a.err, 12, abort))) break;
             ready_ph ^= 1u << s;
+            if (l == 0) {
+              if (!(ok = mbar_wait(b_feat + 8 * s, (feat_ph >> s) & 1u, a.err, 15, abort))) break;
+              feat_ph ^= 1u << s;
+            }
             tc_fence_after();
             const uint32_t d = tmem + (uint32_t)(s * N);
             const uint32_t a_base = smem_u32(act + (size_t)s * ACT_BYTES);
@@ -228,6 +250,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
               }
             }
             if (ok) umma_commit(b_full + 8 * s);
+            if (ok && l == a.L - 1) umma_commit(b_free + 8 * s);
           }
         }
       }
@@ -237,25 +260,46 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
       while (!mbar_test(b_drain, 0) && clock64() - t0 < WAIT_CYCLES) {
       }
     }
+  } else if (warp >= FEATURE_WARP) {
+    const int t = threadIdx.x - 32 * FEATURE_WARP;  // rows t and t + 64
+    const bool aligned = (reinterpret_cast<uintptr_t>(a.x) & 15) == 0;
+    uint32_t free_ph = 0;  // bit s: the parity slot s waits for next
+    bool ok = true;
+    Features f;
+    auto put = [&](int s, long long tile, bool loaded) {
+      unsigned char* as = act + (size_t)s * ACT_BYTES;
+      if (!loaded) load_features(a, tile * BM + t, aligned, f);
+      store_features(as, a, t, f);
+      load_features(a, tile * BM + t + 64, aligned, f);
+      store_features(as, a, t + 64, f);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the MMAs (async proxy)
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_feat + 8 * s);
+    };
+    if ((long long)blockIdx.x < pairs)
+      for (int s = 0; s < 2 && 2 * (long long)blockIdx.x + s < tiles; ++s) put(s, 2 * (long long)blockIdx.x + s, false);
+    for (long long P = blockIdx.x; ok && P < pairs; P += gridDim.x) {
+      const int ns = 2 * P + 1 < tiles ? 2 : 1;
+      const long long Pn = P + gridDim.x;
+      for (int s = 0; s < ns; ++s) {
+        if (Pn >= pairs || 2 * Pn + s >= tiles) continue;  // no next tile for this slot
+        const long long row = (2 * Pn + s) * BM + t;
+        load_features(a, row, aligned, f);  // in flight during the wait
+        if (row + 64 < a.M) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.x + (row + 64) * a.n_in));
+        if (!(ok = mbar_wait(b_free + 8 * s, (free_ph >> s) & 1u, a.err, 16, abort))) break;
+        free_ph ^= 1u << s;
+        put(s, 2 * Pn + s, true);
+      }
+    }
   } else {
     const int q = warp & 3;           // the lane quarter this warp may read
     const int cq = (warp - 2) >> 2;   // its 64-column quarter = one k-block of the next layer
     const int r = q * 32 + lane;      // row within the tile
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     uint32_t full_ph = 0;  // bit s: the parity slot s waits for next
-    FeatureShare fs;
-    // the first pair's features
-    if ((long long)blockIdx.x < pairs) {
-      const long long P = blockIdx.x;
-      const int ns = 2 * P + 1 < tiles ? 2 : 1;
-      for (int s = 0; s < ns; ++s) {
-        load_features(a, (2 * P + s) * BM + r, cq, fs);
-        store_features(act + (size_t)s * ACT_BYTES, a, r, cq, fs);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the MMAs (async proxy)
-        __syncwarp();
-        if (lane == 0) mbar_arrive(b_ready + 8 * s);
-      }
-    }
+    // both accumulators are free for the first pair
+    if ((long long)blockIdx.x < pairs && lane == 0)
+      for (int s = 0; s < 2 && 2 * (long long)blockIdx.x + s < tiles; ++s) mbar_arrive(b_ready + 8 * s);
     bool ok = true;
     for (long long P = blockIdx.x; ok && P < pairs; P += gridDim.x) {
       const int ns = 2 * P + 1 < tiles ? 2 : 1;
@@ -267,7 +311,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
           const long long row = (2 * P + s) * BM + r;
           const bool next = Pn < pairs && 2 * Pn + s < tiles;  // a next tile for this slot
           unsigned char* as = act + (size_t)s * ACT_BYTES;
-          if (last && next) load_features(a, (2 * Pn + s) * BM + r, cq, fs);  // in flight during the head
           // 16 columns at a time, the next 16 in flight (tensor memory, bias)
           // while these are computed; the first bias before the wait
           uint32_t u[2][16];
@@ -361,7 +404,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_infer(const __grid_constant_
               __syncwarp();
               if (lane == 0) head_count[s * 4 + q] = 0;
             }
-            if (next) store_features(as, a, r, cq, fs);
           }
           if (!last || next) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
