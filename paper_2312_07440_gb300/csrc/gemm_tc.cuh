@@ -105,11 +105,17 @@ __device__ __forceinline__ unsigned short bf16_bits(float x) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(x));
 }
 
-// SiLU'(z) = sigma(z) (1 + z (1 - sigma(z))), sigma from the same functions
-__device__ __forceinline__ float dsilu_f(float z) {
+// sigma(z) = 1 / (1 + 2^(-z log2 e)) from the same functions
+__device__ __forceinline__ float sigma_f(float z) {
   float e, s;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(1.0f + e));
+  return s;
+}
+
+// SiLU'(z) = sigma(z) (1 + z (1 - sigma(z)))
+__device__ __forceinline__ float dsilu_f(float z) {
+  const float s = sigma_f(z);
   return s * fmaf(z, 1.0f - s, 1.0f);
 }
 

@@ -183,21 +183,51 @@ __global__ void k_dense_in(const float* __restrict__ X, int B, int nin, const fl
 // and the block's feature rows sit in shared memory, and each thread
 // accumulates 8 rows x 8 consecutive units (64 FMAs per 16 shared loads),
 // then writes 8-unit runs of Z (FP32, when kept) and H (BF16, 16 bytes).
+// pick.n > 0 (training): row r of the batch is row draw(r) of X, whose BF16
+// copy and label go to pick.Xb and pick.yb, instead of three launches (indices,
+// gather, layer).
 constexpr int DI_ROWS = 64, DI_N = 256, DI_MAX_IN = 64;
+struct Pick {
+  uint64_t seed, step;
+  int64_t n;  // rows of X to draw from; 0: take row r as it is
+  const float* y;
+  bf16* Xb;
+  float* yb;
+};
+// minibatch row b: a counter-based hash (splitmix64) of (seed, step, b)
+__device__ __forceinline__ int64_t draw_row(uint64_t seed, uint64_t step, int b, int64_t n) {
+  uint64_t z = seed + 0x9E3779B97F4A7C15ull * (step * 0x100000001ull + (uint64_t)b + 1);
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  z ^= z >> 31;
+  return (int64_t)(z % (uint64_t)n);
+}
 __global__ void __launch_bounds__(256) k_dense_in_256(const float* __restrict__ X, int B, int nin,
                                                       const float* __restrict__ W, const float* __restrict__ b,
-                                                      float* __restrict__ Z, bf16* __restrict__ H) {
+                                                      float* __restrict__ Z, bf16* __restrict__ H, const Pick pick) {
+  __shared__ int64_t src[DI_ROWS];
   extern __shared__ __align__(16) float di_smem[];
   float* Ws = di_smem;                      // [nin][256]
   float* Xs = di_smem + nin * DI_N;         // [DI_ROWS][nin + 1]
   const int ldx = nin + 1;
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   const long long r0 = (long long)blockIdx.x * DI_ROWS;
+  if (tid < DI_ROWS) {
+    const long long r = r0 + tid;
+    src[tid] = r;
+    if (pick.n > 0 && r < B) {
+      src[tid] = draw_row(pick.seed, pick.step, (int)r, pick.n);
+      pick.yb[r] = __ldg(pick.y + src[tid]);
+    }
+  }
   for (int i = tid; i < nin * DI_N / 4; i += 256)
     reinterpret_cast<float4*>(Ws)[i] = __ldg(reinterpret_cast<const float4*>(W) + i);
+  __syncthreads();
   for (int i = tid; i < DI_ROWS * nin; i += 256) {
     const int r = i / nin, k = i % nin;
-    Xs[r * ldx + k] = r0 + r < B ? __ldg(X + (r0 + r) * nin + k) : 0.0f;
+    const float v = r0 + r < B ? __ldg(X + src[r] * nin + k) : 0.0f;
+    Xs[r * ldx + k] = v;
+    if (pick.n > 0 && r0 + r < B) pick.Xb[r0 * nin + i] = f2bf(v);
   }
   __syncthreads();
   float acc[8][8];
@@ -230,8 +260,9 @@ __global__ void __launch_bounds__(256) k_dense_in_256(const float* __restrict__ 
     unsigned hw[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const float z0 = acc[i][2 * j], z1 = acc[i][2 * j + 1];
-      hw[j] = (unsigned)f2bf(z0 * sigmoidf_(z0)) | ((unsigned)f2bf(z1 * sigmoidf_(z1)) << 16);
+      float h0, h1;
+      tcg::silu_pair(tcg::pack2(acc[i][2 * j], acc[i][2 * j + 1]), h0, h1);
+      hw[j] = tcg::bf16x2(h0, h1);
     }
     *reinterpret_cast<uint4*>(H + o) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
   }
@@ -335,14 +366,22 @@ __global__ void __launch_bounds__(32 * HD_WARPS) k_head(const float* __restrict_
     g0[j] = g1[j] = 0.0f;
   }
   const float b0 = b[0], b1 = b[1];
-  for (int r = blockIdx.x * HD_WARPS + warp; r < B; r += gridDim.x * HD_WARPS) {
+  const int rows = gridDim.x * HD_WARPS, first = blockIdx.x * HD_WARPS + warp;
+  float4 na, nb;
+  auto load = [&](int r) {
     const float4* zp = reinterpret_cast<const float4*>(Z + (long long)r * 256 + 8 * l);
-    const float4 za = __ldcs(zp), zb = __ldcs(zp + 1);
+    na = __ldcs(zp);
+    nb = __ldcs(zp + 1);
+  };
+  if (first < B) load(first);
+  for (int r = first; r < B; r += rows) {
+    const float4 za = na, zb = nb;
+    if (r + rows < B) load(r + rows);  // the next row is in flight
     const float z[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
     float s[8], a0 = 0.0f, a1 = 0.0f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      s[j] = sigmoidf_(z[j]);
+      s[j] = tcg::sigma_f(z[j]);
       const float h = z[j] * s[j];
       a0 = fmaf(h, w0[j], a0);
       a1 = fmaf(h, w1[j], a1);
@@ -392,18 +431,28 @@ __global__ void __launch_bounds__(32 * HD_WARPS) k_head(const float* __restrict_
 }
 
 // g[i] = the slices of parameter i added in order: parts [S][stride] below
-// `head`, hparts [HB][HD_PARAMS] for the output layer from there on
-__global__ void k_sum_grads(const float* __restrict__ parts, int S, long long stride, const float* __restrict__ hparts,
-                            int HB, long long head, long long n, float* __restrict__ g) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float* p = i < head ? parts + i : hparts + (i - head);
-  const long long step = i < head ? stride : HD_PARAMS;
-  const int m = i < head ? S : HB;
+// `head`; from there on the output layer's hparts [HB][HD_PARAMS], a warp per
+// parameter (each lane every 32nd block, then a fixed tree)
+__global__ void __launch_bounds__(128) k_sum_grads(const float* __restrict__ parts, int S, long long stride,
+                                                   const float* __restrict__ hparts, int HB, long long head,
+                                                   float* __restrict__ g) {
+  const long long body = (head + 127) / 128;  // blocks of the body
+  if (blockIdx.x < body) {
+    const long long i = (long long)blockIdx.x * 128 + threadIdx.x;
+    if (i >= head) return;
+    float s = 0.0f;
+#pragma unroll 10
+    for (int z = 0; z < S; ++z) s += __ldcg(parts + i + z * stride);
+    g[i] = s;
+    return;
+  }
+  const long long i = (blockIdx.x - body) * 4 + (threadIdx.x >> 5);
+  if (i >= HD_PARAMS) return;
   float s = 0.0f;
-#pragma unroll 8
-  for (int z = 0; z < m; ++z) s += __ldcg(p + z * step);
-  g[i] = s;
+  for (int z = threadIdx.x & 31; z < HB; z += 32) s += __ldcg(hparts + i + (long long)z * HD_PARAMS);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) g[head + i] = s;
 }
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ gr, float* __restrict__ m1,
@@ -426,13 +475,18 @@ __global__ void k_to_bf16(const float* __restrict__ x, bf16* __restrict__ y, lon
   if (i < n) y[i] = f2bf(x[i]);
 }
 
-// BF16 transpose of a K x N FP32 weight matrix: Wt[n][k] = bf16(W[k][n])
-// (the tensor-core GEMM reads the weights K-major)
-__global__ void k_transpose_bf16(const float* __restrict__ W, int K, int N, bf16* __restrict__ Wt) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)K * N) return;
-  const int n = (int)(t / K), k = (int)(t % K);
-  Wt[t] = f2bf(W[(long long)k * N + n]);
+// BF16 transposes of the hidden layers' H x H weights (layer 1 + blockIdx.y at
+// W + blockIdx.y step): Wt[n][k] = bf16(W[k][n]) (the tensor-core GEMM reads
+// the weights K-major), 32 x 32 tiles through shared memory
+__global__ void __launch_bounds__(256) k_transpose_bf16(const float* __restrict__ W, long long step, int H,
+                                                        bf16* __restrict__ Wt) {
+  __shared__ float t[32][33];
+  const int nt = H >> 5, k0 = (blockIdx.x / nt) * 32, n0 = (blockIdx.x % nt) * 32;
+  const float* w = W + blockIdx.y * step;
+  bf16* o = Wt + (long long)blockIdx.y * H * H;
+  for (int i = threadIdx.x; i < 1024; i += 256) t[i >> 5][i & 31] = w[(long long)(k0 + (i >> 5)) * H + n0 + (i & 31)];
+  __syncthreads();
+  for (int i = threadIdx.x; i < 1024; i += 256) o[(long long)(n0 + (i >> 5)) * H + k0 + (i & 31)] = f2bf(t[i & 31][i >> 5]);
 }
 
 // The inference kernel's weights: k-block g, row n, column k of
@@ -475,15 +529,10 @@ __global__ void k_gather_rows(const float* __restrict__ X, const float* __restri
   if (j == 0 && y) yb[b] = y[r];
 }
 
-// minibatch indices: a counter-based hash (splitmix64) of (seed, step, b)
+// minibatch indices
 __global__ void k_batch_indices(uint64_t seed, uint64_t step, int B, int64_t n, int64_t* __restrict__ idx) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  uint64_t z = seed + 0x9E3779B97F4A7C15ull * (step * 0x100000001ull + (uint64_t)b + 1);
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  z ^= z >> 31;
-  idx[b] = (int64_t)(z % (uint64_t)n);
+  if (b < B) idx[b] = draw_row(seed, step, b, n);
 }
 
 }  // namespace
@@ -642,14 +691,14 @@ int launch_gemm_tc(rw_mlp* m, int l, const bf16* A, int B, tcg::Epi e) {
   return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "tensor-core GEMM launch");
 }
 
-// transposed BF16 copies of the hidden weights (after any change of p)
-int refresh_wt(rw_mlp* m) {
+// transposed BF16 copies of the hidden weights (after any change of p) and,
+// unless more training steps follow, the inference kernel's packed weights
+int refresh_wt(rw_mlp* m, bool pack = true) {
   const int H = m->hidden;
   if (m->wt)
-    for (int l = 1; l < m->n_layers; ++l)
-      k_transpose_bf16<<<(unsigned)(((long long)H * H + 255) / 256), 256, 0, m->stream>>>(
-          m->p + m->w_off[l], H, H, m->wt + (size_t)(l - 1) * H * H);
-  if (m->wpack) {
+    k_transpose_bf16<<<dim3((H / 32) * (H / 32), m->n_layers - 1), 256, 0, m->stream>>>(
+        m->p + m->w_off[1], (long long)H * H + H, H, m->wt);
+  if (m->wpack && pack) {
     PackArgs a{};
     for (int l = 0; l < m->n_layers; ++l) a.W[l] = m->p + m->w_off[l];
     a.nin = m->n_in;
@@ -682,18 +731,21 @@ int launch_gemm(rw_mlp* m, int epi, GemmArgs a) {
   return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "gemm launch");
 }
 
+// the input layer's kernel draws and gathers its rows itself
+bool picks_rows(const rw_mlp* m) { return m->hidden == DI_N && m->n_in <= DI_MAX_IN; }
+
 // Forward for B <= max_batch rows of FP32 features xf (device); output in
 // m->out.  First and last layers in FP32, hidden layers BF16 on the tensor
 // cores.  infer: only the output is needed, so the last hidden layer's
 // tensor-core epilogue computes the output layer itself and writes neither
 // its pre-activation nor its activation.  head: false leaves the output layer
 // to the backward pass.
-int forward_batch(rw_mlp* m, const float* xf, int B, bool infer = false, bool head = true) {
+int forward_batch(rw_mlp* m, const float* xf, int B, bool infer = false, bool head = true, const Pick& pick = Pick{}) {
   const int L = m->n_layers;
   const bool tc = tc_usable(m);
   // inference on the tensor-core path reads no pre-activation back
   const bool keep_z = !(infer && tc && L >= 2);
-  if (m->hidden == DI_N && m->n_in <= DI_MAX_IN) {
+  if (picks_rows(m)) {
     const size_t sm = ((size_t)m->n_in * DI_N + (size_t)DI_ROWS * (m->n_in + 1)) * sizeof(float);
     static bool attr = false;
     if (!attr && sm > 48 * 1024) {
@@ -702,7 +754,7 @@ int forward_batch(rw_mlp* m, const float* xf, int B, bool infer = false, bool he
       attr = true;
     }
     k_dense_in_256<<<(unsigned)((B + DI_ROWS - 1) / DI_ROWS), 256, sm, m->stream>>>(
-        xf, B, m->n_in, m->p + m->w_off[0], m->p + m->b_off[0], keep_z ? m->Z[0] : nullptr, m->H[0]);
+        xf, B, m->n_in, m->p + m->w_off[0], m->p + m->b_off[0], keep_z ? m->Z[0] : nullptr, m->H[0], pick);
   } else {
     k_dense_in<<<(unsigned)(((long long)B * m->hidden + 255) / 256), 256, 0, m->stream>>>(
         xf, B, m->n_in, m->p + m->w_off[0], m->p + m->b_off[0], m->hidden, keep_z ? m->Z[0] : nullptr, m->H[0]);
@@ -826,8 +878,8 @@ int backward_tc(rw_mlp* m, const float* y, int B, float inv_tau2, float lam) {
   }
   if (nd >= L && (rc = launch_wgrad_tc(m, 0, L, B))) return rc;
   const int rows = ((B + m->w_slices - 1) / m->w_slices + tcg::wg::ROWS - 1) / tcg::wg::ROWS * tcg::wg::ROWS;
-  k_sum_grads<<<(unsigned)((m->n_params + 127) / 128), 128, 0, m->stream>>>(
-      m->wparts, (B + rows - 1) / rows, m->w_stride, m->hparts, hb, m->w_off[L], m->n_params, m->g);
+  k_sum_grads<<<(unsigned)((m->w_off[L] + 127) / 128 + (HD_PARAMS + 3) / 4), 128, 0, m->stream>>>(
+      m->wparts, (B + rows - 1) / rows, m->w_stride, m->hparts, hb, m->w_off[L], m->g);
   return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "backward launch");
 }
 
@@ -904,10 +956,10 @@ int backward_batch(rw_mlp* m, int B) {
 }
 
 // forward, loss and gradient of B rows (m->X: their BF16 copy) into m->loss, m->g
-int loss_gradient(rw_mlp* m, const float* x, const float* y, int B, float tau, float lam) {
+int loss_gradient(rw_mlp* m, const float* x, const float* y, int B, float tau, float lam, const Pick& pick = Pick{}) {
   const bool tc = backward_tc_usable(m);
   const float inv_tau2 = 1.0f / (tau * tau);
-  int rc = forward_batch(m, x, B, false, !tc);
+  int rc = forward_batch(m, x, B, false, !tc, pick);
   if (rc) return rc;
   if (tc) return backward_tc(m, y, B, inv_tau2, lam);
   k_loss<<<(B + 127) / 128, 128, 0, m->stream>>>(m->out, y, B, inv_tau2, lam, m->dout_f, m->dout_b, m->loss);
@@ -1138,16 +1190,21 @@ int rw_mlp_train(rw_mlp* m, const float* d_x, const float* d_y, int64_t n, int b
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   for (int64_t it = 0; it < n_steps; ++it) {
     const uint64_t step = (uint64_t)m->step;
-    k_batch_indices<<<(batch + 127) / 128, 128, 0, m->stream>>>(seed, step, batch, n, m->idx);
-    k_gather_rows<<<(unsigned)(((long long)batch * m->n_in + 255) / 256), 256, 0, m->stream>>>(
-        d_x, d_y, m->idx, batch, m->n_in, m->Xf, m->X, m->yb);
-    int rc = loss_gradient(m, m->Xf, m->yb, batch, tau, lam);
+    int rc;
+    if (picks_rows(m)) {
+      rc = loss_gradient(m, d_x, m->yb, batch, tau, lam, Pick{seed, step, n, d_y, m->X, m->yb});
+    } else {
+      k_batch_indices<<<(batch + 127) / 128, 128, 0, m->stream>>>(seed, step, batch, n, m->idx);
+      k_gather_rows<<<(unsigned)(((long long)batch * m->n_in + 255) / 256), 256, 0, m->stream>>>(
+          d_x, d_y, m->idx, batch, m->n_in, m->Xf, m->X, m->yb);
+      rc = loss_gradient(m, m->Xf, m->yb, batch, tau, lam);
+    }
     if (rc) return rc;
     m->step += 1;
     const float c1 = 1.0f - powf(b1, (float)m->step), c2 = 1.0f - powf(b2, (float)m->step);
     k_adam<<<(unsigned)((m->n_params + 255) / 256), 256, 0, m->stream>>>(m->p, m->g, m->m1, m->m2, m->pb,
                                                                          m->n_params, lr, b1, b2, eps, c1, c2);
-    if ((rc = refresh_wt(m))) return rc;
+    if ((rc = refresh_wt(m, it + 1 == n_steps))) return rc;
   }
   return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "train launch");
 }
