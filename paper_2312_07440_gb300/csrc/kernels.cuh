@@ -292,6 +292,14 @@ __global__ void __launch_bounds__(256, MINB) k_reweight(const __grid_constant__ 
     for (int i = 0; i < NEXT; ++i)
 #pragma unroll
       for (int m = 0; m < 4; ++m) load_mom(p[i][m], __ldg(a.mom + ((long long)(i * 4 + m)) * a.ld + evc));
+    // the next event's momenta and weight on their way to L2 (g g -> t tbar
+    // FP32, 1,048,576 events, waited for them at every trip: 369 -> 338 us)
+    if (ev + ngroups < E && lane == 0) {
+#pragma unroll
+      for (int i = 0; i < 4 * NEXT; ++i)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.mom + (long long)i * a.ld + ev + ngroups));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(a.w + ev + ngroups));
+    }
     typename Shared<Proc, R, LB>::type common;
     if constexpr (Shared<Proc, R, LB>::value) Proc::template common<R, LB>(p, lane, gmask, common);
     // One call site for every evaluation (original, then each point), so that
