@@ -8,11 +8,12 @@
 // current for each helicity it does not depend on and spills; its unrolled code
 // overflows the instruction cache.  Here the sum takes about half the
 // arithmetic, the code is compact loops over tasks, and 8 (FP64) or 16 (FP32)
-// warps fit an SM.  FP64 is bound by the FP64 pipe (90 % busy, 3.8k warp
-// instructions per evaluation), FP32 by issue and shared-memory latency (2.5
-// of 4 instructions per cycle).  Per call with one point, against the
-// per-thread kernels: FP64 131,072 events 118.1 -> 57.5 ms, FP32 262,147
-// events 15.26 -> 4.28 ms, FP16-mixed 65,536 events 3.94 -> 1.34 ms.
+// warps fit an SM.  FP64 is bound by the FP64 pipe (90 % busy), FP32 by issue,
+// instruction fetch and shared-memory latency (2.5 of 4 instructions per cycle
+// before its warps were kept in step).  Per call with one point, against the
+// per-thread kernels: FP64 131,072 events 118 -> 53.1 ms (57.5 before products
+// of currents were shared between the three- and four-gluon currents), FP32
+// 262,147 events 15.3 -> 3.31 ms, FP16-mixed 65,536 events 3.94 -> 1.13 ms.
 //
 // CM_STORE_*: instead of summing colours, the lanes write their amplitude
 // vectors for the separate tensor-core pass (colour_tc.cuh), one evaluation
@@ -40,8 +41,8 @@ __device__ __forceinline__ df quad_sum(df v) {
 
 // Momenta of up to two evaluations from the event's (W.u.p), moved onto the
 // mass shell where the point's top mass differs: the common 3-momentum scale
-// by Newton's method in FP32, then two FP64 or one double-float step, as in
-// reshuffle_tops (qcd.cuh), particle 2 + (lane & 3) of evaluation
+// by Newton's method in FP32, then two FP64 or one double-float step (compare
+// reshuffle_tops in qcd.cuh), particle 2 + (lane & 3) of evaluation
 // (lane >> 2) & 1 in each lane.  Returns whether evaluation b's masses fit, in
 // bit b.
 template <class R>
@@ -182,15 +183,21 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_coop(const __gr
       }
       __syncwarp();
 #pragma unroll 1
+      for (int t = lane; t < nb * N_DOT; t += 32) {
+        const int b = t >= N_DOT, i = t - b * N_DOT;
+        W.product(b, i, words[TW_DOT + i]);
+      }
+      __syncwarp();
+#pragma unroll 1
       for (int t = lane; t < nb * N_J3; t += 32) {
-        const int b = t >= N_J3;
-        W.three_gluons(b, t - b * N_J3, words[TW_J3 + t - b * N_J3]);
+        const int b = t >= N_J3, i = t - b * N_J3;
+        W.three_gluons(b, i, words[TW_J3 + i], words[TW_J3B + i]);
       }
       __syncwarp();
 #pragma unroll 1
       for (int t = lane; t < nb * N_J4; t += 32) {
-        const int b = t >= N_J4;
-        W.four_gluons(b, t - b * N_J4, words[TW_J4 + t - b * N_J4], words[TW_J4B + t - b * N_J4]);
+        const int b = t >= N_J4, i = t - b * N_J4;
+        W.four_gluons(b, i, words[TW_J4 + i], words[TW_J4B + i], words[TW_J4C + i], words[TW_J4D + i]);
       }
 #pragma unroll 1
       for (int b = 0; b < nb; ++b) {

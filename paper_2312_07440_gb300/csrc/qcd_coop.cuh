@@ -134,6 +134,15 @@ struct Warp {
       for (int m = 0; m < 4; ++m) *reinterpret_cast<double2*>(a + m * N_OBJ * 16) = make_double2(v.c[m].r, v.c[m].i);
     }
   }
+  // the products of currents (complex numbers): in the work spinors' first
+  // chunks, which are free until the gluon currents are done
+  __device__ __forceinline__ cx<R> prod(int b, int i) const {
+    return *reinterpret_cast<const cx<R>*>(obj + (b * N_OBJ + O_WK + i) * 16);
+  }
+  __device__ __forceinline__ cx<R> prod(int b, int i, unsigned neg) const {
+    const cx<R> v = prod(b, i);
+    return {flip(v.r, neg), flip(v.i, neg)};
+  }
   __device__ __forceinline__ cv<R> vec(int i) const { return get<cv<R>>(i); }
   __device__ __forceinline__ sp<R> spin(int i) const { return get<sp<R>>(i); }
   // the generated code's operands: work spinors, S(g), T(g)
@@ -193,16 +202,28 @@ struct Warp {
           put(ob + O_E + 2 * l - 1, e[0]);
           put(ob + O_E + 2 * l, e[1]);
         }
-      } else if (l == 4) {
-        sp<R> x[2];
-        ubar_out<R>(p, R(m), x);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) put(ob + O_X0 + 2 + h, sp<R>{{x[h].c[2], x[h].c[3], x[h].c[0], x[h].c[1]}});
       } else {
-        sp<R> x[2];
-        v_out<R>(p, R(m), x);
-        put(ob + O_X0, x[0]);
-        put(ob + O_X0 + 1, x[1]);
+        // the top's ub (swapped) and the antitop's v from the same pieces:
+        // u(+) = (w- chi+, w+ chi+), u(-) = (w+ chi-, w- chi-), ub = (u_R*, u_L*)
+        // and v(+) = (w+ chi-, -w- chi-), v(-) = (w- chi+, -w+ chi+)
+        cx<R> cp[2], cm[2];
+        const R pp = chi_pm(p, cp, cm);
+        R wp, wm;
+        omegas(p[0], pp, R(m), wp, wm);
+        const bool top = l == 4;
+        const R f[2] = {top ? wm : wp, top ? wp : wm}, g[2] = {top ? wp : -wm, top ? wm : -wp};
+        const unsigned neg = top ? 0x80000000u : 0u;  // conjugated
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          sp<R> x;
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const cx<R> c = top == (h == 0) ? cp[i] : cm[i];
+            x.c[i] = {f[h] * c.r, flip(f[h] * c.i, neg)};
+            x.c[2 + i] = {g[h] * c.r, flip(g[h] * c.i, neg)};
+          }
+          put(ob + O_X0 + (top ? 2 : 0) + h, x);
+        }
       }
     }
   }
@@ -289,7 +310,13 @@ struct Warp {
     put(ob + O_J2 + t, o);
   }
 
-  __device__ __forceinline__ void three_gluons(int b, int t, unsigned w) {
+  __device__ __forceinline__ void product(int b, int t, unsigned w) {
+    const int ob = b * N_EV;
+    const cv<R> A = vec(ob + O_E + (w & 7)), B = vec(ob + ((w >> 3) & 1 ? O_J2 : O_E) + ((w >> 4) & 31));
+    *reinterpret_cast<cx<R>*>(obj + (b * N_OBJ + O_WK + t) * 16) = dot(A, B);
+  }
+
+  __device__ __forceinline__ void three_gluons(int b, int t, unsigned w, unsigned w2) {
     const int ob = b * N_EV;
     const cv<R> A = vec(ob + O_E + (w & 7)), B = vec(ob + O_E + ((w >> 3) & 7)), C = vec(ob + O_E + ((w >> 6) & 7));
     const cv<R> AB = flip(vec(ob + O_J2 + ((w >> 9) & 31)), (w >> 14) << 31);
@@ -297,7 +324,8 @@ struct Warp {
     const int ma = 1 << ((w >> 21) & 3), mb = 1 << ((w >> 23) & 3), mc = 1 << ((w >> 25) & 3);
     const Kin& K = kin[b];
     const R c = -K.ik2[ma | mb | mc];
-    const cx<R> ab = dot(A, B), bc = dot(B, C), ac = dot(A, C), pa = dot(A, BC), pc = dot(AB, C);
+    const cx<R> ab = prod(b, w2 & 31), bc = prod(b, (w2 >> 5) & 31), ac = prod(b, (w2 >> 10) & 31);
+    const cx<R> pa = prod(b, (w2 >> 15) & 127, (w >> 20) << 31), pc = prod(b, (w2 >> 22) & 127, (w >> 14) << 31);
     const cx<R> fa = c * (bc - p_dot(K, ma, BC)), fc = c * (ab + p_dot(K, mc, AB));
     const cx<R> fb = (R(-2) * c) * ac;
     const cx<R> fbc = c * p_dot(K, mb | mc, A), fab = (-c) * p_dot(K, ma | mb, C);
@@ -318,31 +346,26 @@ struct Warp {
 
   // (ub gamma v).J(0bcd) for the four spin states of the pair; the parts of the
   // current along its own momentum drop out (ub gamma v is conserved)
-  __device__ __forceinline__ void four_gluons(int b, int t, unsigned w, unsigned w2) {
+  __device__ __forceinline__ void four_gluons(int b, int t, unsigned w, unsigned w2, unsigned w3, unsigned w4) {
     const int ob = b * N_EV;
     const Kin& K = kin[b];
     const int gb = (w >> 26) & 3, gc = (w >> 28) & 3, gd = (w2 >> 12) & 3;
     const int mb = 1 << gb, mc = 1 << gc, md = 1 << gd;
+    const unsigned nbc = (w >> 19) << 31, ncd = (w >> 25) << 31;
     const cv<R> A = vec(ob + O_E), B = vec(ob + O_E + (w & 7)), C = vec(ob + O_E + ((w >> 3) & 7)),
                 D = vec(ob + O_E + ((w >> 6) & 7));
-    const cx<R> ab = dot(A, B), ad = dot(A, D), cd = dot(C, D);
-    cx<R> fa, fb, fc, fd, fab, fcd, fbc, fabc, fbcd, ga, gab, gabc;
+    cx<R> fa = prod(b, (w3 >> 15) & 127, nbc) + prod(b, w4 & 127, ncd);          // BC.D + B.CD
+    cx<R> fd = prod(b, (w3 >> 22) & 127, nbc) + prod(b, (w4 >> 14) & 127);       // A.BC + AB.C
+    const cx<R> ad = prod(b, (w3 >> 5) & 31), acd = prod(b, (w4 >> 7) & 127, ncd), abd = prod(b, (w4 >> 21) & 127);
+    const cx<R> fbc = {R(-2) * ad.r, R(-2) * ad.i}, fb = {R(-2) * acd.r, R(-2) * acd.i},
+                fc = {R(-2) * abd.r, R(-2) * abd.i};
+    cx<R> fab, fcd, fabc, fbcd, ga, gab, gabc;
     {
-      const cv<R> BC = flip(vec(ob + O_J2 + ((w >> 14) & 31)), (w >> 19) << 31);
-      fa = dot(BC, D);
-      fd = dot(A, BC);
-      fbc = {R(-2) * ad.r, R(-2) * ad.i};
-    }
-    {
-      const cv<R> AB = vec(ob + O_J2 + ((w >> 9) & 31)), CD = flip(vec(ob + O_J2 + ((w >> 20) & 31)), (w >> 25) << 31);
-      fa = fa + dot(B, CD);
-      fd = fd + dot(AB, C);
-      const cx<R> x = dot(A, CD), y = dot(AB, D), z = dot(AB, CD);
-      fb = {R(-2) * x.r, R(-2) * x.i};
-      fc = {R(-2) * y.r, R(-2) * y.i};
+      const cv<R> AB = vec(ob + O_J2 + ((w >> 9) & 31)), CD = flip(vec(ob + O_J2 + ((w >> 20) & 31)), ncd);
+      const cx<R> z = dot(AB, CD);
       gab = z + z;
-      fab = cd - p_dot(K, 1 | mb, CD);
-      fcd = ab + p_dot(K, mc | md, AB);
+      fab = prod(b, (w3 >> 10) & 31) - p_dot(K, 1 | mb, CD);
+      fcd = prod(b, w3 & 31) + p_dot(K, mc | md, AB);
     }
     {
       const cv<R> BCD = vec(ob + O_J3 + ((w2 >> 6) & 63));
@@ -374,8 +397,8 @@ struct Warp {
     add(C, fc);
     add(D, fd);
     add(vec(ob + O_J2 + ((w >> 9) & 31)), fab);
-    add(flip(vec(ob + O_J2 + ((w >> 14) & 31)), (w >> 19) << 31), fbc);
-    add(flip(vec(ob + O_J2 + ((w >> 20) & 31)), (w >> 25) << 31), fcd);
+    add(flip(vec(ob + O_J2 + ((w >> 14) & 31)), nbc), fbc);
+    add(flip(vec(ob + O_J2 + ((w >> 20) & 31)), ncd), fcd);
     add(vec(ob + O_J3 + (w2 & 63)), fabc);
     add(vec(ob + O_J3 + ((w2 >> 6) & 63)), fbcd);
     const R c = -K.ik2[15];

@@ -78,6 +78,19 @@ def j3_of(seq, h):
     raise KeyError(seq)
 
 
+def ee_idx(a, b, h):
+    """Index of E_a.E_b among the products."""
+    return j2_idx(a, b, h)[0]
+
+
+def ej_idx(i, j, k, h):
+    """Index of E_i.J(jk) among the products, up to the sign of the order j, k (as j2_idx)."""
+    st = tuple(sorted((i, j, k)))
+    t, w = SETS.index(st), st.index(i)
+    hh = 2 * h[st[1]] + h[st[2]] if t < 3 else 4 * h[1] + 2 * h[2] + h[3]
+    return N_J2 + 12 * t + (4 if t < 3 else 8) * w + hh
+
+
 def x1_idx(g, h, lam):
     """S(g) or T(g) within its 14 spinors."""
     return lam if g == 0 else 2 + (g - 1) * 4 + h[g] * 2 + lam
@@ -98,24 +111,44 @@ def tasks():
     out = {}
     # J(ab): E_a, E_b, gluons a, b
     out["J2"] = [bits([(e_idx(a, h), 3), (e_idx(b, h), 3), (a, 2), (b, 2)]) for a, b in PAIRS for h in hels((a, b))]
-    # J(abc): E_a, E_b, E_c, J(ab), sign, J(bc), sign, gluons
-    j3 = {}
+    # products of currents that several three- and four-gluon currents need: E_a.E_b, then E_i.J(jk):
+    # E, whether the other is a J, its index
+    d = {}
+    for a, b in PAIRS:
+        for h in hels((a, b)):
+            d[ee_idx(a, b, h)] = bits([(e_idx(a, h), 3), (0, 1), (e_idx(b, h), 5)])
+    for st in SETS:
+        for i in st:
+            j, k = [g for g in st if g != i]
+            for h in hels(st):
+                d[ej_idx(i, j, k, h)] = bits([(e_idx(i, h), 3), (1, 1), (j2_idx(j, k, h)[0], 5)])
+    assert sorted(d) == list(range(len(d)))
+    out["DOT"] = [d[i] for i in range(len(d))]
+    # J(abc), two words: E_a, E_b, E_c, J(ab), sign, J(bc), sign, gluons | products ab, bc, ac, a.bc, c.ab
+    j3, j3b = {}, {}
     for t, o, (a, b, c) in J3_ORDERS:
         for h in hels(SETS[t]):
             (ab, sab), (bc, sbc) = j2_idx(a, b, h), j2_idx(b, c, h)
             j3[j3_idx(t, o, h)] = bits([(e_idx(a, h), 3), (e_idx(b, h), 3), (e_idx(c, h), 3), (ab, 5), (sab, 1), (bc, 5),
                                         (sbc, 1), (a, 2), (b, 2), (c, 2)])
+            j3b[j3_idx(t, o, h)] = bits([(ee_idx(a, b, h), 5), (ee_idx(b, c, h), 5), (ee_idx(a, c, h), 5),
+                                         (ej_idx(a, b, c, h), 7), (ej_idx(c, a, b, h), 7)])
     assert sorted(j3) == list(range(N_J3))
-    out["J3"] = [j3[i] for i in range(N_J3)]
-    # J(0bcd), two words: E_b, E_c, E_d, J(0b), J(bc), sign, J(cd), sign, gluons b, c | J(0bc), J(bcd), sign, gluon d
-    lo, hi = [], []
+    out["J3"], out["J3B"] = [j3[i] for i in range(N_J3)], [j3b[i] for i in range(N_J3)]
+    # J(0bcd), four words: E_b, E_c, E_d, J(0b), J(bc), sign, J(cd), sign, gluons b, c | J(0bc), J(bcd), gluon d |
+    # products 0b, 0d, cd, d.bc, 0.bc | b.cd, 0.cd, c.0b, d.0b
+    lo, hi, pc, pd = [], [], [], []
     for b, c, d in PERMS:
         for h in hels((1, 2, 3)):
             (ob, _), (bc, sbc), (cd, scd) = j2_idx(0, b, h), j2_idx(b, c, h), j2_idx(c, d, h)
             lo.append(bits([(e_idx(b, h), 3), (e_idx(c, h), 3), (e_idx(d, h), 3), (ob, 5), (bc, 5), (sbc, 1), (cd, 5),
                             (scd, 1), (b, 2), (c, 2)]))
             hi.append(bits([(j3_of((0, b, c), h), 6), (j3_of((b, c, d), h), 6), (d, 2)]))
-    out["J4"], out["J4B"] = lo, hi
+            pc.append(bits([(ee_idx(0, b, h), 5), (ee_idx(0, d, h), 5), (ee_idx(c, d, h), 5), (ej_idx(d, b, c, h), 7),
+                            (ej_idx(0, b, c, h), 7)]))
+            pd.append(bits([(ej_idx(b, c, d, h), 7), (ej_idx(0, c, d, h), 7), (ej_idx(c, 0, b, h), 7),
+                            (ej_idx(d, 0, b, h), 7)]))
+    out["J4"], out["J4B"], out["J4C"], out["J4D"] = lo, hi, pc, pd
     # S(g), then T(g): E, spinor (0, 1 v; 2, 3 ub), propagator mask
     x1 = [None] * 28
     for side in (0, 1):
@@ -316,7 +349,7 @@ def emit():
     T = tasks()
     at = 0
     words = []
-    for k in ("J2", "J3", "J4", "J4B", "X1", "R3", "Y", "X2"):
+    for k in ("J2", "DOT", "J3", "J3B", "J4", "J4B", "J4C", "J4D", "X1", "R3", "Y", "X2"):
         w(f"constexpr int TW_{k} = {at}, N_{k} = {len(T[k])};")
         words += T[k]
         at += len(T[k])
