@@ -117,6 +117,8 @@ def source_sha(process, mode):
     if not os.path.exists(os.path.join(d, tu)):
         tu = f"proc_{process}.cu"
     tus = {tu, "rw_abi.cu"}
+    if process == "gg_ttgg":
+        tus.add("proc_gg_ttgg_coop.cu")
     if mode.startswith("mixed"):  # the separate colour pass's translation units
         tus |= {fn for fn in os.listdir(d) if fn.startswith(f"proc_{process}_store_") and fn.endswith(".cu")}
     for fn in sorted(os.listdir(d)):
@@ -325,19 +327,22 @@ def evaluations(process, pts):
     return len({float(q[1]) for q in [p0, *pts]})
 
 
-def alu_roofline(info, E, pts, t_step, mode, peaks, workload):
+def alu_roofline(info, E, pts, t_step, mode, peaks, workload, lane_bits):
     """Roofline of the fused kernel against the plain-ALU pipe it is bound by:
     algorithmic flops = the launch's distinct evaluations x the generator's
     static count of one helicity sum per event; the ncu-executed count beside
     it when a profile of the current sources records one."""
+    from paper_2312_07440_gb300.gen import coop_gen
     P = len(pts)
-    flops_event = evaluations(ev.WORKLOADS[workload].process, pts) * info.flops_hel_sum
+    per_warp = lane_bits == 5  # one warp per event (g g -> t tbar g g)
+    flops_event = evaluations(ev.WORKLOADS[workload].process, pts) * (
+        coop_gen.flops_per_evaluation() if per_warp else info.flops_hel_sum)
     achieved = E * flops_event / t_step / 1e12
     pipe = "fp64" if mode == "fp64" else "fp32"
     peak = peaks[pipe]
-    kernel = "k_reweight (fused: amplitudes, colour sum, helicity sum, ratio, W', sigma)"
+    kernel = ("k_coop" if per_warp else "k_reweight") + " (fused: amplitudes, colour sum, helicity sum, ratio, W', sigma)"
     if mode.startswith("mixed") and workload == "gg_ttgg_1m" and P <= 3:
-        kernel = ("k_amp_store (amplitudes, J vectors stored in 16 bits; the executed count and traffic are its own) "
+        kernel = ("k_coop" if per_warp else "k_amp_store") + (" (amplitudes, J vectors stored in 16 bits; the executed count and traffic are its own) "
                   "+ k_colour_tc (tcgen05 colour pass, HBM-bound), per step")
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": profiled_value(workload, mode, "dram_bytes_per_launch"),
@@ -499,7 +504,7 @@ def run_ours(args):
     if not args.no_e2e:
         e2e = run_e2e(ctx, torch, dev, mom_h, w_h, E, P, N, world, args)
     info = rwgt.process_info(wl.process)
-    roof = alu_roofline(info, E, pts, t_step, args.mode, peaks, wl.name)
+    roof = alu_roofline(info, E, pts, t_step, args.mode, peaks, wl.name, lane_bits)
     ctx.close()
     del ws
 
@@ -583,7 +588,7 @@ def run_variant(torch, rwgt, dev, stream, wl, variant, mode, sample, args, flush
            "point_set": f"{variant}: {POINT_SETS.get(variant, variant)}", "mode": mode,
            "value": E * P / t, "unit": UNIT, "ms_per_step": 1e3 * t, "dtype": DTYPE[mode],
            "tuning": {"lane_bits": lb, "block": bl},
-           "roofline": alu_roofline(info, E, pts, t, mode, peaks, wl.name),
+           "roofline": alu_roofline(info, E, pts, t, mode, peaks, wl.name, lb),
            "accuracy_vs_oracle": accuracy_sample(wl, pts, mom_h, w_h, wn, mode, n=n_acc, variant=variant)}
     if variant == "default" and wl.process in ("gg_ttg", "gg_ttgg"):
         out["r_is_exactly_one"] = bool(torch.all(wn == w.unsqueeze(0)).item())

@@ -260,9 +260,8 @@ __global__ void __launch_bounds__(256) k_dense_in_256(const float* __restrict__ 
     unsigned hw[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      float h0, h1;
-      tcg::silu_pair(tcg::pack2(acc[i][2 * j], acc[i][2 * j + 1]), h0, h1);
-      hw[j] = tcg::bf16x2(h0, h1);
+      const float z0 = acc[i][2 * j], z1 = acc[i][2 * j + 1];
+      hw[j] = (unsigned)f2bf(z0 * sigmoidf_(z0)) | ((unsigned)f2bf(z1 * sigmoidf_(z1)) << 16);
     }
     *reinterpret_cast<uint4*>(H + o) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
   }
@@ -345,11 +344,12 @@ __global__ void k_loss(const float* __restrict__ out, const float* __restrict__ 
 }
 
 // Output layer, loss and their backward for hidden = 256, one warp per row and
-// eight units per lane: out = SiLU(Z) W + b and the loss as in k_dense_out and
-// k_loss, dZ = bf16(dOut W^T SiLU'(Z)), and per block the sums over its rows of
-// dW [256][2] (BF16 activations and errors) and db [2]: hparts [blocks][514].
-// One pass over Z (16 MB for 16,384 rows) instead of three, and one launch
-// instead of seven (16 us instead of 73).
+// units l + 32 j in lane l: out = SiLU(Z) W + b and the loss as in k_dense_out
+// and k_loss (the same arithmetic in the same order, as BF16 roundings of dZ
+// hang on it), dZ = bf16(dOut W^T SiLU'(Z)), and per block the sums over its
+// rows of dW [256][2] (BF16 activations and errors) and db [2]: hparts
+// [blocks][514].  One pass over Z (16 MB for 16,384 rows) instead of three, and
+// one launch instead of seven (73 us).
 constexpr int HD_WARPS = 16, HD_PARAMS = 2 * 256 + 2;
 __global__ void __launch_bounds__(32 * HD_WARPS) k_head(const float* __restrict__ Z, const float* __restrict__ y, int B,
                                                         const float* __restrict__ W, const float* __restrict__ b,
@@ -360,28 +360,27 @@ __global__ void __launch_bounds__(32 * HD_WARPS) k_head(const float* __restrict_
   float w0[8], w1[8], g0[8], g1[8], e0 = 0.0f, e1 = 0.0f;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const float2 v = reinterpret_cast<const float2*>(W)[8 * l + j];
+    const float2 v = reinterpret_cast<const float2*>(W)[l + 32 * j];
     w0[j] = v.x;
     w1[j] = v.y;
     g0[j] = g1[j] = 0.0f;
   }
   const float b0 = b[0], b1 = b[1];
   const int rows = gridDim.x * HD_WARPS, first = blockIdx.x * HD_WARPS + warp;
-  float4 na, nb;
+  float n[8];
   auto load = [&](int r) {
-    const float4* zp = reinterpret_cast<const float4*>(Z + (long long)r * 256 + 8 * l);
-    na = __ldcs(zp);
-    nb = __ldcs(zp + 1);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) n[j] = __ldcs(Z + (long long)r * 256 + l + 32 * j);
   };
   if (first < B) load(first);
   for (int r = first; r < B; r += rows) {
-    const float4 za = na, zb = nb;
+    float z[8], s[8], a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) z[j] = n[j];
     if (r + rows < B) load(r + rows);  // the next row is in flight
-    const float z[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
-    float s[8], a0 = 0.0f, a1 = 0.0f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      s[j] = tcg::sigma_f(z[j]);
+      s[j] = sigmoidf_(z[j]);
       const float h = z[j] * s[j];
       a0 = fmaf(h, w0[j], a0);
       a1 = fmaf(h, w1[j], a1);
@@ -392,20 +391,27 @@ __global__ void __launch_bounds__(32 * HD_WARPS) k_head(const float* __restrict_
       a1 += __shfl_xor_sync(0xffffffffu, a1, o);
     }
     const float mu = a0 + b0, q = fminf(fmaxf(a1 + b1, -16.0f), 4.0f);
-    const float res = y[r] - mu, e2 = __expf(-2.0f * q);
-    const float dmu = -2.0f * res * inv_tau2 / B, ds = lam * (1.0f - res * res * e2) / B;
+    const float res = y[r] - mu;
+    const float e2 = __expf(-2.0f * q);
+    const float dmu = -2.0f * res * inv_tau2 / B;
+    const float ds = lam * (1.0f - res * res * e2) / B;
     const float dmu_b = bf2f(f2bf(dmu)), ds_b = bf2f(f2bf(ds));
-    unsigned hw[4];
+    unsigned d[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const float hb = bf2f(f2bf(z[j] * s[j]));
       g0[j] = fmaf(hb, dmu_b, g0[j]);
       g1[j] = fmaf(hb, ds_b, g1[j]);
       const float dh = dmu * w0[j] + ds * w1[j];
-      const unsigned d = f2bf(dh * s[j] * (1.0f + z[j] * (1.0f - s[j])));
-      hw[j >> 1] = j & 1 ? hw[j >> 1] | (d << 16) : d;
+      d[j] = f2bf(dh * s[j] * (1.0f + z[j] * (1.0f - s[j])));
     }
-    *reinterpret_cast<uint4*>(dZ + (long long)r * 256 + 8 * l) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+    // pairs of units in one word: even lanes take those of an even j, odd lanes of the next
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) {
+      const unsigned other = __shfl_xor_sync(0xffffffffu, l & 1 ? d[j] : d[j + 1], 1);
+      const unsigned w = l & 1 ? other | (d[j + 1] << 16) : d[j] | (other << 16);
+      *reinterpret_cast<unsigned*>(dZ + (long long)r * 256 + 32 * (j + (l & 1)) + (l & ~1)) = w;
+    }
     if (l == 0) {
       e0 += dmu;
       e1 += ds;
@@ -414,8 +420,8 @@ __global__ void __launch_bounds__(32 * HD_WARPS) k_head(const float* __restrict_
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    sums[warp][2 * (8 * l + j)] = g0[j];
-    sums[warp][2 * (8 * l + j) + 1] = g1[j];
+    sums[warp][2 * (l + 32 * j)] = g0[j];
+    sums[warp][2 * (l + 32 * j) + 1] = g1[j];
   }
   if (l == 0) {
     sums[warp][512] = e0;
@@ -883,7 +889,14 @@ int backward_tc(rw_mlp* m, const float* y, int B, float inv_tau2, float lam) {
   return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "backward launch");
 }
 
-bool backward_tc_usable(const rw_mlp* m) { return m->wparts && m->n_layers >= 2 && tc_usable(m); }
+// From 2,048 rows on: there a last-bit difference in a gradient's sum vanishes
+// in the average over the batch.  Below, it turns enough BF16 roundings in the
+// steps that follow to move the first moments by 2.6e-5 over 16 steps of 1,000
+// rows (7e-6 with 4,096), so small batches keep the row-by-row sums' order.
+constexpr int WG_MIN_ROWS = 2048;
+bool backward_tc_usable(const rw_mlp* m, int B) {
+  return m->wparts && m->n_layers >= 2 && B >= WG_MIN_ROWS && tc_usable(m);
+}
 
 // Backward: gradients of the loss (m->dout_f set, m->X holds the BF16
 // inputs) into m->g.  Weight gradients on the tensor cores (BF16 operands,
@@ -957,7 +970,7 @@ int backward_batch(rw_mlp* m, int B) {
 
 // forward, loss and gradient of B rows (m->X: their BF16 copy) into m->loss, m->g
 int loss_gradient(rw_mlp* m, const float* x, const float* y, int B, float tau, float lam, const Pick& pick = Pick{}) {
-  const bool tc = backward_tc_usable(m);
+  const bool tc = backward_tc_usable(m, B);
   const float inv_tau2 = 1.0f / (tau * tau);
   int rc = forward_batch(m, x, B, false, !tc, pick);
   if (rc) return rc;

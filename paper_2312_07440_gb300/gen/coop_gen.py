@@ -337,6 +337,25 @@ def colour_blocks():
     return blocks
 
 
+def flops_per_evaluation():
+    """Floating-point operations of one helicity and colour sum (FMA = 2; the set-up is not counted)."""
+    F = qcd_gen.FLOPS
+    t = {k: len(v) for k, v in tasks().items()}
+    n = 4 * F["fcur"] + t["J2"] * F["current2"] + t["DOT"] * F["dot"]
+    n += t["J3"] * (F["current3"] - 5 * F["dot"])
+    # four gluons: three more products, six momentum products, nine currents and three momenta combined, four
+    # products with the quark line's current
+    n += t["J4"] * (3 * F["dot"] + 6 * 16 + 20 + 9 * 32 + 40 + 4 * (F["dot"] + 2))
+    n += t["X1"] * (F["slash"] + F["fprop"]) + (t["R3"] + t["Y"]) * F["slash"]
+    n += t["X2"] * (2 * F["slash"] + F["sp_add"]) + t["X2"] // 2 * F["fprop"]
+    lane = sum(F["rowcol"] + 2 * len(tg) for _, dots in steps() for _, _, tg in dots)
+    lane += sum(2 * (len(v) - 1) for v in w_terms().values())
+    lane += 2 * 2 * (8 * 3 + 4 * 2)  # butterflies: two orbits of eight, two of four
+    for rows, L, D in colour_blocks():
+        lane += sum(4 for r in L for x in r if x) + 5 * len(D)
+    return n + 32 * lane
+
+
 def emit():
     lines = []
     w = lines.append
