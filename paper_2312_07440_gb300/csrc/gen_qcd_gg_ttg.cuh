@@ -40,6 +40,13 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
     const ws<R> W0 = weyl_form(E0);
     const sp<R> T0_0 = row_prop(Kn.qc[6], Kn.mc[6], row_slash(W0, X.ub[0]));
     const sp<R> T0_1 = row_prop(Kn.qc[6], Kn.mc[6], row_slash(W0, X.ub[1]));
+    // the quark line's currents and (below) the spinors of gluons 0 and 1 for both antitop
+    // helicities at the level they depend on, in local memory, instead of once per inner trip
+    // (200,003 events x 2 points FP64 15.03 -> 13.57 ms, 131,072 x 64 FP32 6.84 -> 6.59 ms)
+    constexpr bool HV = LB < 3, H1 = LB < 2;
+    cv<R> VC[HV ? 4 : 1];
+    if constexpr (HV)
+      for (int i = 0; i < 4; ++i) VC[i] = fcur(X.ub[i & 1], X.v[i >> 1]);
     [[maybe_unused]] sp<R> S_0v0, S_0v1;
     if constexpr (LB < 3) {
       S_0v0 = fprop(Kn.qc[1], Kn.mc[1], slash(W0, X.v[0]));
@@ -54,6 +61,17 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
       const sp<R> T1_1 = row_prop(Kn.qc[5], Kn.mc[5], row_slash(W1, X.ub[1]));
       cv<R> J0_1 = current2(E0, Kn.P[1], E1, Kn.P[2], Kn.cg[3]);
       const cv<R> J1_0 = neg(J0_1);
+      sp<R> S1v[H1 ? 2 : 1], X01v[H1 ? 2 : 1], X10v[H1 ? 2 : 1];
+      if constexpr (H1) {
+        const ws<R> WJ = weyl_form(J0_1);
+        for (int i = 0; i < 2; ++i) {
+          S1v[i] = fprop(Kn.qc[2], Kn.mc[2], slash(W1, X.v[i]));
+          X01v[i] = slash(WJ, X.v[i]);
+          X10v[i] = spneg(X01v[i]);
+          slash_acc(X01v[i], W0, S1v[i]);
+          slash_acc(X10v[i], W1, i ? S_0v1 : S_0v0);
+        }
+      }
       #pragma unroll 1
       for (int i2 = 0; i2 < (LB >= 2 ? 1 : 2); ++i2) {
         const int h2 = LB >= 2 ? ((lane >> (LB - 2)) & 1) : i2;
@@ -76,22 +94,31 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
           sp<R> S_0;
           if constexpr (LB < 3) S_0 = h3 ? S_0v1 : S_0v0;
           else S_0 = fprop(Kn.qc[1], Kn.mc[1], slash(W0, S_E));
-          const sp<R> S_1 = fprop(Kn.qc[2], Kn.mc[2], slash(W1, S_E));
+          sp<R> S_1;
+          if constexpr (H1) S_1 = S1v[h3];
+          else S_1 = fprop(Kn.qc[2], Kn.mc[2], slash(W1, S_E));
           const sp<R> S_2 = fprop(Kn.qc[4], Kn.mc[4], slash(W2, S_E));
           cx<R> A0_0, A0_1, A1_0, A1_1, A2_0, A2_1, A3_0, A3_1, A4_0, A4_1, A5_0, A5_1;
           {
-            const ws<R> WJ = weyl_form(J0_1);
-            sp<R> x = slash(WJ, S_E), y = spneg(x);  // J(01) v and J(10) v
-            slash_acc(x, W0, S_1);
-            slash_acc(y, W1, S_0);
+            sp<R> x, y;  // J(01) v and J(10) v, then the single-gluon terms
+            if constexpr (H1) {
+              x = X01v[h3];
+              y = X10v[h3];
+            } else {
+              x = slash(weyl_form(J0_1), S_E);
+              y = spneg(x);
+              slash_acc(x, W0, S_1);
+              slash_acc(y, W1, S_0);
+            }
             A4_0 = rowcol(T2_0, x);
             A5_0 = rowcol(T2_0, y);
             A4_1 = rowcol(T2_1, x);
             A5_1 = rowcol(T2_1, y);
           }
           {
-            const ws<R> WJ = weyl_form(J0_2);
-            sp<R> x = slash(WJ, S_E), y = spneg(x);  // J(02) v and J(20) v
+            sp<R> x, y;  // J(02) v and J(20) v, then the single-gluon terms
+            x = slash(weyl_form(J0_2), S_E);
+            y = spneg(x);
             slash_acc(x, W0, S_2);
             slash_acc(y, W2, S_0);
             A2_0 = rowcol(T1_0, x);
@@ -100,8 +127,9 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
             A3_1 = rowcol(T1_1, y);
           }
           {
-            const ws<R> WJ = weyl_form(J1_2);
-            sp<R> x = slash(WJ, S_E), y = spneg(x);  // J(12) v and J(21) v
+            sp<R> x, y;  // J(12) v and J(21) v, then the single-gluon terms
+            x = slash(weyl_form(J1_2), S_E);
+            y = spneg(x);
             slash_acc(x, W1, S_2);
             slash_acc(y, W2, S_1);
             A0_0 = rowcol(T0_0, x);
@@ -137,7 +165,9 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
             A5_1 = A5_1 - d1;
           }
           {
-            const cv<R> V = fcur(X.ub[0], S_E);
+            cv<R> V;
+            if constexpr (HV) V = VC[2 * h3 + 0];
+            else V = fcur(X.ub[0], S_E);
             const cx<R> u = dot(V, J0_1_2), t = dot(V, J0_2_1), m = u + t;
             A0_0 = A0_0 + u;
             A5_0 = A5_0 + u;
@@ -147,7 +177,9 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
             A4_0 = A4_0 - m;
           }
           {
-            const cv<R> V = fcur(X.ub[1], S_E);
+            cv<R> V;
+            if constexpr (HV) V = VC[2 * h3 + 1];
+            else V = fcur(X.ub[1], S_E);
             const cx<R> u = dot(V, J0_1_2), t = dot(V, J0_2_1), m = u + t;
             A0_1 = A0_1 + u;
             A5_1 = A5_1 + u;
@@ -218,5 +250,5 @@ __device__ __forceinline__ R hel_sum(const QcdExt<R, NG>& X, const QcdKin<R, NG>
 }
 
 // floating-point operations of one full helicity sum (all levels, all loop trips)
-constexpr long FLOPS_HEL_SUM = 23073;
+constexpr long FLOPS_HEL_SUM = 20969;
 }}  // namespace

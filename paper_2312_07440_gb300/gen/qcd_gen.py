@@ -219,25 +219,38 @@ def emit_cut(w, ind, n, em, jref):
     w(f"{ind}sp<R> S_0;")
     w(f"{ind}if constexpr (LB < {n}) S_0 = h{n} ? S_0v1 : S_0v0;")
     w(f"{ind}else S_0 = fprop(Kn.qc[1], Kn.mc[1], slash(W0, S_E));")
-    for g in (1, 2):
-        w(f"{ind}const sp<R> S_{g} = fprop(Kn.qc[{1 << g}], Kn.mc[{1 << g}], slash(W{g}, S_E));")
-    em.count(n, "slash_w", 2)
-    em.count(n, "fprop", 2)
+    w(f"{ind}sp<R> S_1;")
+    w(f"{ind}if constexpr (H1) S_1 = S1v[h{n}];")
+    w(f"{ind}else S_1 = fprop(Kn.qc[2], Kn.mc[2], slash(W1, S_E));")
+    w(f"{ind}const sp<R> S_2 = fprop(Kn.qc[4], Kn.mc[4], slash(W2, S_E));")
+    em.count(n, "slash_w")
+    em.count(n, "fprop")
     k = {p: i for i, p in enumerate(perms)}
     w(f"{ind}cx<R> {', '.join(f'A{i}_{h}' for i in range(len(perms)) for h in (0, 1))};")
     for b, c in ((0, 1), (0, 2), (1, 2)):
         a = 3 - b - c
         w(f"{ind}{{")
-        w(f"{ind}  const ws<R> WJ = weyl_form({jref((b, c))});")
-        w(f"{ind}  sp<R> x = slash(WJ, S_E), y = spneg(x);  // J({b}{c}) v and J({c}{b}) v")
-        w(f"{ind}  slash_acc(x, W{b}, S_{c});")
-        w(f"{ind}  slash_acc(y, W{c}, S_{b});")
+        w(f"{ind}  sp<R> x, y;  // J({b}{c}) v and J({c}{b}) v, then the single-gluon terms")
+        form = [f"x = slash(weyl_form({jref((b, c))}), S_E);", "y = spneg(x);", f"slash_acc(x, W{b}, S_{c});",
+                f"slash_acc(y, W{c}, S_{b});"]
+        if (b, c) == (0, 1):
+            w(f"{ind}  if constexpr (H1) {{")
+            w(f"{ind}    x = X01v[h{n}];")
+            w(f"{ind}    y = X10v[h{n}];")
+            w(f"{ind}  }} else {{")
+            for f in form:
+                w(f"{ind}    {f}")
+            w(f"{ind}  }}")
+        else:
+            for f in form:
+                w(f"{ind}  {f}")
         for h in (0, 1):
             w(f"{ind}  A{k[a, b, c]}_{h} = rowcol(T{a}_{h}, x);")
             w(f"{ind}  A{k[a, c, b]}_{h} = rowcol(T{a}_{h}, y);")
-        em.count(n, "weyl")
-        em.count(n, "slash_w", 3)
-        em.count(n, "sp_add", 2)
+        if (b, c) != (0, 1):
+            em.count(n, "weyl")
+            em.count(n, "slash_w", 3)
+            em.count(n, "sp_add", 2)
         em.count(n, "rowcol", 4)
         w(f"{ind}}}")
     for a, b in ((0, 1), (0, 2), (1, 2)):
@@ -254,12 +267,13 @@ def emit_cut(w, ind, n, em, jref):
         w(f"{ind}}}")
     for h in (0, 1):
         w(f"{ind}{{")
-        w(f"{ind}  const cv<R> V = fcur(X.ub[{h}], S_E);")
+        w(f"{ind}  cv<R> V;")
+        w(f"{ind}  if constexpr (HV) V = VC[2 * h{n} + {h}];")
+        w(f"{ind}  else V = fcur(X.ub[{h}], S_E);")
         w(f"{ind}  const cx<R> u = dot(V, J0_1_2), t = dot(V, J0_2_1), m = u + t;")
         for p, e in (((0, 1, 2), "+ u"), ((2, 1, 0), "+ u"), ((0, 2, 1), "+ t"), ((1, 2, 0), "+ t"), ((1, 0, 2), "- m"),
                      ((2, 0, 1), "- m")):
             w(f"{ind}  A{k[p]}_{h} = A{k[p]}_{h} {e};")
-        em.count(n, "fcur")
         em.count(n, "dot", 2)
         em.count(n, "cadd", 7)
         w(f"{ind}}}")
@@ -403,6 +417,15 @@ def emit_process(name, n, outgoing_gluons, n_identical, hoist_weyl=True, share_f
             w(f"{ind}const sp<R> T{g}_1 = row_prop(Kn.qc[{m}], Kn.mc[{m}], row_slash(W{g}, X.ub[1]));")
             em.count(g, "slash_w", 2)
             em.count(g, "fprop", 2)
+            if g == 0:
+                w(f"{ind}// the quark line's currents and (below) the spinors of gluons 0 and 1 for both antitop")
+                w(f"{ind}// helicities at the level they depend on, in local memory, instead of once per inner trip")
+                w(f"{ind}// (200,003 events x 2 points FP64 15.03 -> 13.57 ms, 131,072 x 64 FP32 6.84 -> 6.59 ms)")
+                w(f"{ind}constexpr bool HV = LB < {n}, H1 = LB < {n - 1};")
+                em.count(g, "fcur", 4)
+                w(f"{ind}cv<R> VC[HV ? 4 : 1];")
+                w(f"{ind}if constexpr (HV)")
+                w(f"{ind}  for (int i = 0; i < 4; ++i) VC[i] = fcur(X.ub[i & 1], X.v[i >> 1]);")
         if g == 0 and hoist_weyl:
             # S(0) depends on the antitop helicity and on gluon 0's, which is
             # fixed: both antitop variants are formed here once instead of at
@@ -466,6 +489,22 @@ def emit_process(name, n, outgoing_gluons, n_identical, hoist_weyl=True, share_f
                     wform[sq] = f"W{nm}"
                     w(f"{ind}const ws<R> W{nm} = weyl_form({nm});")
                     em.count(g, "weyl")
+        if cut and g == 1:
+            em.count(g, "weyl")
+            em.count(g, "slash_w", 8)
+            em.count(g, "sp_add", 4)
+            em.count(g, "fprop", 2)
+            w(f"{ind}sp<R> S1v[H1 ? 2 : 1], X01v[H1 ? 2 : 1], X10v[H1 ? 2 : 1];")
+            w(f"{ind}if constexpr (H1) {{")
+            w(f"{ind}  const ws<R> WJ = weyl_form(J0_1);")
+            w(f"{ind}  for (int i = 0; i < 2; ++i) {{")
+            w(f"{ind}    S1v[i] = fprop(Kn.qc[2], Kn.mc[2], slash(W1, X.v[i]));")
+            w(f"{ind}    X01v[i] = slash(WJ, X.v[i]);")
+            w(f"{ind}    X10v[i] = spneg(X01v[i]);")
+            w(f"{ind}    slash_acc(X01v[i], W0, S1v[i]);")
+            w(f"{ind}    slash_acc(X10v[i], W1, i ? S_0v1 : S_0v0);")
+            w(f"{ind}  }}")
+            w(f"{ind}}}")
     # antitop level: the fermion currents psi(rho) = S_rho (rho a proper
     # sequence of gluons attached from the antitop end), the amputated spinor
     # X(sigma) = sum_c Jslash(sigma[..c]) psi(sigma[c+1..]) of every ordering and
