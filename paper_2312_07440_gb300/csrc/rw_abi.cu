@@ -335,23 +335,29 @@ int lane_bits_for(const rw_ctx* c, int kind) {
   return lb < 5 || registry().find(c->process, c->mode, lb, kind) ? lb : per_thread_lane_bits(c->mode);
 }
 
-// Threads per block: the caller's choice, else 128.  The warp-per-event kernels
-// (32 lanes) run 8 warps per block, so that the shared memory left beside the
-// task tables holds the most warps an SM can have, unless there are too few
-// events to give every SM that many: then 2, which spreads them over the SMs.
-int block_for(const rw_ctx* c, int lb, long long E) {
+size_t smem_bytes(const KernelEntry* k, int block, int npts) {
+  return (size_t)k->smem_per_thread * block + (size_t)(block / 32) * npts * k->smem_per_warp_point;
+}
+
+// Threads per block of a launch with npts sums: the caller's choice, else 128.
+// The warp-per-event kernels (32 lanes) run 8 warps per block, so that the
+// shared memory left beside the task tables holds the most warps an SM can
+// have; 4 where the sums of many points leave no room for 8; and 2 when there
+// are too few events to give every SM that many, which spreads them over the SMs.
+int block_for(const rw_ctx* c, const KernelEntry* k, long long E, int npts) {
   if (c->block > 0) return c->block;
-  if (lb < 5) return 128;
-  return E >= 16LL * c->sm_count ? 256 : 64;
+  if (!k || k->lane_bits < 5) return 128;
+  if (E < 16LL * c->sm_count) return 64;
+  return c->smem_optin > 0 && smem_bytes(k, 256, npts) + static_smem(k->func) > (size_t)c->smem_optin ? 128 : 256;
 }
 
 int shape(rw_ctx* c, int P, long long E, Shape& sh) {
   const int lb = lane_bits_for(c, 0);
   const KernelEntry* k = registry().find(c->process, c->mode, lb);
   if (!k) return fail(c, RW_ERR_MODE, "no kernel for process %d mode %d lane_bits %d", c->process, c->mode, lb);
-  const int block = block_for(c, lb, E);
+  const int block = block_for(c, k, E, P + 1);
   if (block > k->max_block) return fail(c, RW_ERR_ARG, "block %d above this variant's %d", block, k->max_block);
-  const size_t smem = (size_t)k->smem_per_thread * block + (size_t)(block / 32) * (P + 1) * k->smem_per_warp_point;
+  const size_t smem = smem_bytes(k, block, P + 1);
   const size_t smem_total = smem + static_smem(k->func);
   if (c->smem_optin > 0 && smem_total > (size_t)c->smem_optin)
     return fail(c, RW_ERR_ARG,
@@ -377,7 +383,7 @@ int shape(rw_ctx* c, int P, long long E, Shape& sh) {
 
 // the amplitude pass, then the tensor-core colour pass (colour_tc.cuh)
 int launch_deferred(rw_ctx* c, RwArgs& a, const KernelEntry* d) {
-  const int block = block_for(c, d->lane_bits, a.E);
+  const int block = block_for(c, d, a.E, 0);
   const int lanes = 1 << d->lane_bits;
   if (block > d->max_block || lanes > block) return fail(c, RW_ERR_ARG, "block %d does not fit this variant", block);
   const size_t smem = (size_t)d->smem_per_thread * block;  // no sums in this pass
@@ -627,7 +633,9 @@ int rw_get_tuning(const rw_ctx* c, int* lane_bits, int* block) {
   if (!c || !lane_bits || !block) return RW_ERR_NULL;
   if (c->process < 0) return RW_ERR_STATE;
   *lane_bits = c->lane_bits >= 0 ? c->lane_bits : default_lane_bits(c->process, c->mode);
-  *block = block_for(c, *lane_bits, c->mom ? c->E : int64_t(1) << 40);
+  const KernelEntry* k = registry().find(c->process, c->mode, *lane_bits);
+  *block = block_for(c, k ? k : registry().find(c->process, c->mode, *lane_bits, 2), c->mom ? c->E : int64_t(1) << 40,
+                     (int)c->pts.size() + 1);
   return RW_OK;
 }
 
@@ -1060,9 +1068,9 @@ extern "C" int rw_reweight_noalloc(rw_ctx* c, const double* d_mom, const double*
   const int lb = lane_bits_for(c, 0);
   const KernelEntry* k = registry().find(c->process, c->mode, lb);
   if (!k) return noalloc_fail(c, RW_ERR_MODE, "no kernel");
-  const int block = block_for(c, lb, E);
+  const int block = block_for(c, k, E, P + 1);
   if (block > k->max_block) return noalloc_fail(c, RW_ERR_ARG, "block too large");
-  const size_t smem = (size_t)k->smem_per_thread * block + (size_t)(block / 32) * (P + 1) * k->smem_per_warp_point;
+  const size_t smem = smem_bytes(k, block, P + 1);
   if (c->smem_optin > 0 && smem + static_smem(k->func) > (size_t)c->smem_optin)
     return noalloc_fail(c, RW_ERR_ARG, "block too large");
   if (ensure_smem(k->func, smem) != cudaSuccess) {
@@ -1672,7 +1680,7 @@ int rw_reweight_interp(rw_ctx* c, int n_nodes, double tol, double* d_wnew, unsig
   cudaError_t e = cudaMemsetAsync(ia.counts, 0, 16, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "memset");
   {
-    const int block = block_for(c, lb, E);
+    const int block = block_for(c, k, E, 0);
     if (block > k->max_block) return fail(c, RW_ERR_ARG, "block %d above this variant's %d", block, k->max_block);
     const size_t ismem = (size_t)k->smem_per_thread * block;
     if (c->smem_optin > 0 && ismem + static_smem(k->func) > (size_t)c->smem_optin)

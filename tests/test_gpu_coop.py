@@ -75,6 +75,18 @@ def test_many_points_and_masses_that_do_not_fit(mode, tol):
     assert g["n_bad"] == t["n_bad"] == 0
 
 
+@pytest.mark.parametrize("mode", ["fp64", "fp32"])
+@pytest.mark.parametrize("P", [64, 70, 256])
+def test_default_launch_fits_every_number_of_points(mode, P):
+    """Enough events for the largest default block, and up to the most points: the sums of many points leave less room
+    beside the warps' memory; the same results as a small block's."""
+    n = 16 * torch.cuda.get_device_properties(DEV).multi_processor_count + 3
+    mom, w = ev.generate(ev.WORKLOADS["gg_ttgg_1m"], n, start=100)
+    pts = np.stack([ev.param_vector(m_t=175.0 if j % 3 else 173.0, alpha_s=0.1 + 1e-4 * j) for j in range(P)])
+    g, t = run(mode, mom, w, pts, lane_bits=-1), run(mode, mom, w, pts, block=64)
+    assert np.array_equal(g["wnew"], t["wnew"]) and np.array_equal(g["me"], t["me"])
+
+
 @pytest.mark.parametrize("mode", ["mixed_fp16"])
 def test_mixed_amplitude_pass(mode):
     """The amplitude pass of the separate colour sum in the warp-per-event form: the same rounding to 16 bits, so within
