@@ -3,8 +3,8 @@
 // the hot path: |M_h|^2 = (Re J)^T C (Re J) + (Im J)^T C (Im J), C = C_int/den
 // real and symmetric).
 //
-// k_amp_store runs the helicity amplitudes exactly as the FP32 mode does (same
-// set-up, same current recursion, same launch shapes), but instead of summing
+// The amplitude pass runs the FP32 helicity amplitudes (MIXED_FP16: one warp per
+// event, coop_kernel.cuh; MIXED_BF16: k_amp_store, 8 lanes), but instead of summing
 // colours it writes every colour-ordered amplitude vector J (the K complex
 // amplitudes of one event, parameter point and helicity) to global memory as
 // two real rows, Re J and Im J, of K FP16 or BF16 values scaled by 2^-e so
