@@ -58,7 +58,7 @@ __device__ __forceinline__ unsigned momenta(Warp<R>& W, int lane, const PointDev
   bool fits = true;
   if (pt0.reshuffle || pt1.reshuffle) {
     mom p2, etot, mi2;
-    float etf, pf, m2f;
+    float etf, pf, m2f, gap;
     if constexpr (sizeof(R) == 8) {
       p2 = p[1] * p[1] + p[2] * p[2] + p[3] * p[3];
       etot = quad_sum(p[0]);
@@ -67,27 +67,48 @@ __device__ __forceinline__ unsigned momenta(Warp<R>& W, int lane, const PointDev
       etf = float(etot);
       pf = float(p2);
       m2f = float(mi2);
+      gap = float(etot - 2.0 * mt);
     } else {
       p2 = df_norm3(p);
       etot = quad_sum(p[0]);
       const df mtd = df_from_double(mt);
       mi2 = part < 2 ? df_mul(mtd, mtd) : df{0.0f, 0.0f};
-      fits = df_sub(etot, df_scale(mtd, 2.0f)).hi > 0.0f;
+      gap = df_sub(etot, df_scale(mtd, 2.0f)).hi;
+      fits = gap > 0.0f;
       etf = etot.hi;
       pf = p2.hi;
       m2f = mi2.hi;
     }
     // a lane's group stops by itself, so an evaluation does not depend on its neighbour in the warp
-    float xf = 1.0f;
+    float xf = 1.0f, slope = 0.0f;
     bool live = fits && moved;
     for (int it = 0; it < 40; ++it) {
       const float r = rsqrtf(m2f + xf * xf * pf);
       const float f = quad_sum((m2f + xf * xf * pf) * r) - etf, d = quad_sum(xf * pf * r);
       float step = __fdividef(f, d);
       if (xf - step <= 0.0f) step = 0.5f * xf;
-      if (live) xf -= step;
+      if (live) {
+        xf -= step;
+        slope = d;
+      }
       live = live && fabsf(step) > 1e-6f * xf;  // the next step would be below FP32's precision
       if (!__any_sync(0xffffffffu, live)) break;
+    }
+    // near the pair threshold in kinetic energies, as shell_scale (qcd.cuh)
+    live = fits && moved && etf > 4.0f * slope * xf;
+    if (__any_sync(0xffffffffu, live)) {
+      const float mf = sqrtf(m2f);
+      if (live) xf = 1.0f;
+#pragma unroll 1
+      for (int it = 0; it < 40; ++it) {
+        const float k = xf * xf * pf, r = rsqrtf(m2f + k);
+        const float f = quad_sum(__fdividef(k, fmaf(m2f + k, r, mf))) - gap, d = quad_sum(xf * pf * r);
+        float step = __fdividef(f, d);
+        if (xf - step <= 0.0f) step = 0.5f * xf;
+        if (live) xf -= step;
+        live = live && fabsf(step) > 1e-6f * xf;
+        if (!__any_sync(0xffffffffu, live)) break;
+      }
     }
     if constexpr (sizeof(R) == 8) {
       double xi = xf, e = 0.0;

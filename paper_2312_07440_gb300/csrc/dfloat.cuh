@@ -82,6 +82,14 @@ __device__ __forceinline__ df df_mul_f(df x, float y) {
 // multiplication by a power of two is exact
 __device__ __forceinline__ df df_scale(df x, float pow2) { return {__fmul_rn(x.hi, pow2), __fmul_rn(x.lo, pow2)}; }
 
+// the float quotient and its remainder's, the remainder exact by FMA; the
+// relative error is a few u^2 and the reciprocal's error squared
+__device__ __forceinline__ df df_div(df x, df y) {
+  const float r = __fdividef(1.0f, y.hi), q = __fmul_rn(x.hi, r);
+  const float e = __fmaf_rn(-q, y.lo, __fadd_rn(__fmaf_rn(-q, y.hi, x.hi), x.lo));
+  return df_fast_two_sum(q, __fmul_rn(e, r));
+}
+
 // x >= 0; one Newton correction of the correctly rounded float root:
 // r = s + (x - s^2) / (2 s), with x - s^2 formed exactly by FMA.
 __device__ __forceinline__ df df_sqrt(df x) {
