@@ -117,7 +117,11 @@ int rw_set_params(rw_ctx* ctx, const rw_params* orig);
 /* Steps 4/7: P modified parameter points (1 <= P <= RW_MAX_POINTS). */
 int rw_set_reweight_points(rw_ctx* ctx, const rw_params* pts, int P);
 /* Launch shape: lanes per event = 2^lane_bits (-1 = default), threads per
-   block (multiple of 32, <= 256; 0 = default). */
+   block (multiple of 32, <= 256; 0 = default).  A block set together with
+   lanes is for the kernels of those lanes: a call that was not compiled for
+   them (the interpolation and the fused mixed modes at 32 lanes) runs its own
+   default shape.  With 32 lanes the block shrinks where the points' sums do
+   not fit beside it. */
 int rw_set_tuning(rw_ctx* ctx, int lane_bits, int block);
 
 /* The launch shape in use (after rw_set_tuning or rw_autotune). */
@@ -129,8 +133,9 @@ int rw_get_tuning(const rw_ctx* ctx, int* lane_bits, int* block);
    NULL).  Events must be loaded.  cache_path (may be NULL): a JSON-lines file of
    {"key": "<gpu>|<process>|<mode>|P<points>|E<2^k>", "lane_bits", "block", "ms"};
    a matching entry is used without timing, a new result is appended.
-   Synchronises the stream; results are unchanged by the choice (every variant
-   computes the same sums; the sigma reduction order follows the grid). */
+   Synchronises the stream.  Every variant computes the same sums; the results
+   of different lanes differ in the rounding of the mode, and the sigma
+   reduction order follows the grid. */
 int rw_autotune(rw_ctx* ctx, int64_t max_events, const char* cache_path, double* ms);
 
 /* Device workspace needed for E events with the current points (bytes).  In

@@ -339,16 +339,32 @@ size_t smem_bytes(const KernelEntry* k, int block, int npts) {
   return (size_t)k->smem_per_thread * block + (size_t)(block / 32) * npts * k->smem_per_warp_point;
 }
 
+// Whether the caller's block was meant for this kernel.  A block chosen together
+// with lanes is not, where those lanes were not compiled and another kernel runs
+// instead (the warp-per-event kernels' 256 threads do not fit the per-thread
+// ones), or where only the separate colour pass's kernel of those lanes takes it.
+bool block_chosen(const rw_ctx* c, const KernelEntry* k) {
+  if (c->block <= 0) return false;
+  if (c->lane_bits < 0) return true;
+  if (k->lane_bits != c->lane_bits) return false;
+  const KernelEntry* d = registry().find(c->process, c->mode, c->lane_bits, 2);
+  return c->block <= k->max_block || !d || c->block > d->max_block;
+}
+
 // Threads per block of a launch with npts sums: the caller's choice, else 128.
-// The warp-per-event kernels (32 lanes) run 8 warps per block, so that the
-// shared memory left beside the task tables holds the most warps an SM can
-// have; 4 where the sums of many points leave no room for 8; and 2 when there
-// are too few events to give every SM that many, which spreads them over the SMs.
+// The warp-per-event kernels (32 lanes) run 8 warps per block, 2 when there are
+// too few events to give every SM that many, which spreads them over the SMs;
+// and fewer than that, or than the caller's choice, where the sums of many
+// points leave no room for it: the points may be set after the choice.
 int block_for(const rw_ctx* c, const KernelEntry* k, long long E, int npts) {
-  if (c->block > 0) return c->block;
-  if (!k || k->lane_bits < 5) return 128;
-  if (E < 16LL * c->sm_count) return 64;
-  return c->smem_optin > 0 && smem_bytes(k, 256, npts) + static_smem(k->func) > (size_t)c->smem_optin ? 128 : 256;
+  const bool chosen = block_chosen(c, k);
+  if (k->lane_bits < 5) return chosen ? c->block : 128;
+  int block = chosen ? c->block : E < 16LL * c->sm_count ? 64 : 256;
+  const int step = chosen ? 32 : block / 2;
+  while (block > step && c->smem_optin > 0 &&
+         smem_bytes(k, block, npts) + static_smem(k->func) > (size_t)c->smem_optin)
+    block -= step;
+  return block;
 }
 
 int shape(rw_ctx* c, int P, long long E, Shape& sh) {
@@ -634,8 +650,8 @@ int rw_get_tuning(const rw_ctx* c, int* lane_bits, int* block) {
   if (c->process < 0) return RW_ERR_STATE;
   *lane_bits = c->lane_bits >= 0 ? c->lane_bits : default_lane_bits(c->process, c->mode);
   const KernelEntry* k = registry().find(c->process, c->mode, *lane_bits);
-  *block = block_for(c, k ? k : registry().find(c->process, c->mode, *lane_bits, 2), c->mom ? c->E : int64_t(1) << 40,
-                     (int)c->pts.size() + 1);
+  if (!k) k = registry().find(c->process, c->mode, *lane_bits, 2);
+  *block = c->block > 0 || !k ? c->block : block_for(c, k, c->mom ? c->E : int64_t(1) << 40, (int)c->pts.size() + 1);
   return RW_OK;
 }
 
