@@ -646,13 +646,6 @@ int launch_mlp_infer(rw_mlp* m, const float* x, long long n, float* out) {
   CUtensorMap tw;
   if (!bf16_map(&tw, m->wpack, (long long)(m->kb0 + 4 * (L - 1)) * 256, tcg::BK, 256))
     return mlp_fail(m, RW_ERR_CUDA, "tensor map encoding");
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(tcg::k_mlp_infer, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tcg::inf::SMEM_BYTES) != cudaSuccess)
-      return mlp_fail(m, RW_ERR_CUDA, "inference kernel shared memory attribute");
-    attr = true;
-  }
   tcg::InferArgs a{};
   a.x = x;
   for (int l = 0; l < L; ++l) a.bias[l] = m->p + m->b_off[l];
@@ -679,13 +672,6 @@ int launch_gemm_tc(rw_mlp* m, int l, const bf16* A, int B, tcg::Epi e) {
   const bf16* Bop = e.Zin ? m->pb + m->w_off[l] : m->wt + (size_t)(l - 1) * H * H;
   if (!bf16_map(&ta, A, B, H, tcg::BM) || !bf16_map(&tb, Bop, H, H, H))
     return mlp_fail(m, RW_ERR_CUDA, "tensor map encoding");
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(tcg::k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcg::SMEM_BYTES) !=
-        cudaSuccess)
-      return mlp_fail(m, RW_ERR_CUDA, "tensor-core GEMM shared memory attribute");
-    attr = true;
-  }
   e.bias = m->p + m->b_off[l];
   e.err = m->tc_err;
   e.M = B;
@@ -740,6 +726,21 @@ int launch_gemm(rw_mlp* m, int epi, GemmArgs a) {
 // the input layer's kernel draws and gathers its rows itself
 bool picks_rows(const rw_mlp* m) { return m->hidden == DI_N && m->n_in <= DI_MAX_IN; }
 
+size_t dense_in_smem(int n_in) { return ((size_t)n_in * DI_N + (size_t)DI_ROWS * (n_in + 1)) * sizeof(float); }
+
+// The limits on dynamic shared memory of the kernels a model launches.  They
+// belong to a function in one device's context, so every model sets them in its
+// own, once.
+bool raise_smem_limits(const rw_mlp* m) {
+  auto raise = [](const void* f, size_t bytes) {
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+  };
+  return (!picks_rows(m) || raise((const void*)k_dense_in_256, dense_in_smem(DI_MAX_IN))) &&
+         (!m->wt || raise((const void*)tcg::k_gemm_tc, tcg::SMEM_BYTES)) &&
+         (!m->wparts || raise((const void*)tcg::wg::k_wgrad_tc, tcg::wg::SMEM_BYTES)) &&
+         (!m->wpack || raise((const void*)tcg::k_mlp_infer, tcg::inf::SMEM_BYTES));
+}
+
 // Forward for B <= max_batch rows of FP32 features xf (device); output in
 // m->out.  First and last layers in FP32, hidden layers BF16 on the tensor
 // cores.  infer: only the output is needed, so the last hidden layer's
@@ -752,13 +753,7 @@ int forward_batch(rw_mlp* m, const float* xf, int B, bool infer = false, bool he
   // inference on the tensor-core path reads no pre-activation back
   const bool keep_z = !(infer && tc && L >= 2);
   if (picks_rows(m)) {
-    const size_t sm = ((size_t)m->n_in * DI_N + (size_t)DI_ROWS * (m->n_in + 1)) * sizeof(float);
-    static bool attr = false;
-    if (!attr && sm > 48 * 1024) {
-      if (cudaFuncSetAttribute(k_dense_in_256, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess)
-        return mlp_fail(m, RW_ERR_CUDA, "first-layer shared memory attribute");
-      attr = true;
-    }
+    const size_t sm = dense_in_smem(m->n_in);
     k_dense_in_256<<<(unsigned)((B + DI_ROWS - 1) / DI_ROWS), 256, sm, m->stream>>>(
         xf, B, m->n_in, m->p + m->w_off[0], m->p + m->b_off[0], keep_z ? m->Z[0] : nullptr, m->H[0], pick);
   } else {
@@ -844,13 +839,6 @@ int launch_wgrad_tc(rw_mlp* m, int l0, int l1, int B) {
     y.K = m->din[l];
     y.item0 = a.n_items;
     a.n_items += (m->din[l] + 127) / 128;
-  }
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(tcg::wg::k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tcg::wg::SMEM_BYTES) != cudaSuccess)
-      return mlp_fail(m, RW_ERR_CUDA, "weight-gradient shared memory attribute");
-    attr = true;
   }
   a.N = H;
   a.B = B;
@@ -1074,6 +1062,7 @@ int rw_mlp_create(rw_mlp** out, int device, void* stream, int n_in, int hidden, 
     ok = ok && dalloc(&m->wparts, (size_t)m->w_slices * m->w_stride) &&
          dalloc(&m->hparts, (size_t)m->head_blocks * HD_PARAMS);
   }
+  ok = ok && raise_smem_limits(m);
   if (ok) {
     k_to_bf16<<<(unsigned)((off + 255) / 256), 256, 0, m->stream>>>(m->p, m->pb, off);
     ok = refresh_wt(m) == RW_OK && cudaStreamSynchronize(m->stream) == cudaSuccess;
