@@ -683,22 +683,26 @@ int launch_gemm_tc(rw_mlp* m, int l, const bf16* A, int B, tcg::Epi e) {
   return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "tensor-core GEMM launch");
 }
 
-// transposed BF16 copies of the hidden weights (after any change of p) and,
-// unless more training steps follow, the inference kernel's packed weights
-int refresh_wt(rw_mlp* m, bool pack = true) {
+// transposed BF16 copies of the hidden weights (after any change of p)
+int transpose_weights(rw_mlp* m) {
   const int H = m->hidden;
   if (m->wt)
     k_transpose_bf16<<<dim3((H / 32) * (H / 32), m->n_layers - 1), 256, 0, m->stream>>>(
         m->p + m->w_off[1], (long long)H * H + H, H, m->wt);
-  if (m->wpack && pack) {
-    PackArgs a{};
-    for (int l = 0; l < m->n_layers; ++l) a.W[l] = m->p + m->w_off[l];
-    a.nin = m->n_in;
-    a.kb0 = m->kb0;
-    a.n_kb = m->kb0 + 4 * (m->n_layers - 1);
-    k_pack_infer<<<(unsigned)(((long long)a.n_kb * 256 * 64 + 255) / 256), 256, 0, m->stream>>>(a, m->wpack);
-  }
   return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "weight transpose");
+}
+
+// and the inference kernel's packed weights
+int refresh_wt(rw_mlp* m) {
+  const int rc = transpose_weights(m);
+  if (rc || !m->wpack) return rc;
+  PackArgs a{};
+  for (int l = 0; l < m->n_layers; ++l) a.W[l] = m->p + m->w_off[l];
+  a.nin = m->n_in;
+  a.kb0 = m->kb0;
+  a.n_kb = m->kb0 + 4 * (m->n_layers - 1);
+  k_pack_infer<<<(unsigned)(((long long)a.n_kb * 256 * 64 + 255) / 256), 256, 0, m->stream>>>(a, m->wpack);
+  return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "weight packing");
 }
 
 // the tensor-core kernels' error flag (a wait that gave up); synchronises
@@ -972,6 +976,28 @@ bool dalloc(T** p, size_t n) {
   return cudaMalloc(reinterpret_cast<void**>(p), n * sizeof(T)) == cudaSuccess;
 }
 
+// One Adam step; last: nothing follows that would make the inference kernel's weights again
+int train_step(rw_mlp* m, const float* d_x, const float* d_y, int64_t n, int batch, float lr, float tau, float lam,
+               uint64_t seed, bool last) {
+  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  const uint64_t step = (uint64_t)m->step;
+  int rc;
+  if (picks_rows(m)) {
+    rc = loss_gradient(m, d_x, m->yb, batch, tau, lam, Pick{seed, step, n, d_y, m->X, m->yb});
+  } else {
+    k_batch_indices<<<(batch + 127) / 128, 128, 0, m->stream>>>(seed, step, batch, n, m->idx);
+    k_gather_rows<<<(unsigned)(((long long)batch * m->n_in + 255) / 256), 256, 0, m->stream>>>(
+        d_x, d_y, m->idx, batch, m->n_in, m->Xf, m->X, m->yb);
+    rc = loss_gradient(m, m->Xf, m->yb, batch, tau, lam);
+  }
+  if (rc) return rc;
+  m->step += 1;
+  const float c1 = 1.0f - powf(b1, (float)m->step), c2 = 1.0f - powf(b2, (float)m->step);
+  k_adam<<<(unsigned)((m->n_params + 255) / 256), 256, 0, m->stream>>>(m->p, m->g, m->m1, m->m2, m->pb, m->n_params,
+                                                                       lr, b1, b2, eps, c1, c2);
+  return last ? refresh_wt(m) : transpose_weights(m);
+}
+
 }  // namespace
 
 extern "C" {
@@ -1189,26 +1215,15 @@ int rw_mlp_train(rw_mlp* m, const float* d_x, const float* d_y, int64_t n, int b
   if (!d_x || !d_y) return mlp_fail(m, RW_ERR_NULL, "NULL buffer");
   if (n <= 0 || batch <= 0 || batch > m->max_batch || n_steps < 0) return mlp_fail(m, RW_ERR_ARG, "bad sizes");
   cudaSetDevice(m->device);
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  for (int64_t it = 0; it < n_steps; ++it) {
-    const uint64_t step = (uint64_t)m->step;
-    int rc;
-    if (picks_rows(m)) {
-      rc = loss_gradient(m, d_x, m->yb, batch, tau, lam, Pick{seed, step, n, d_y, m->X, m->yb});
-    } else {
-      k_batch_indices<<<(batch + 127) / 128, 128, 0, m->stream>>>(seed, step, batch, n, m->idx);
-      k_gather_rows<<<(unsigned)(((long long)batch * m->n_in + 255) / 256), 256, 0, m->stream>>>(
-          d_x, d_y, m->idx, batch, m->n_in, m->Xf, m->X, m->yb);
-      rc = loss_gradient(m, m->Xf, m->yb, batch, tau, lam);
-    }
-    if (rc) return rc;
-    m->step += 1;
-    const float c1 = 1.0f - powf(b1, (float)m->step), c2 = 1.0f - powf(b2, (float)m->step);
-    k_adam<<<(unsigned)((m->n_params + 255) / 256), 256, 0, m->stream>>>(m->p, m->g, m->m1, m->m2, m->pb,
-                                                                         m->n_params, lr, b1, b2, eps, c1, c2);
-    if ((rc = refresh_wt(m, it + 1 == n_steps))) return rc;
-  }
-  return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "train launch");
+  int rc = RW_OK;
+  for (int64_t it = 0; it < n_steps && rc == RW_OK; ++it)
+    rc = train_step(m, d_x, d_y, n, batch, lr, tau, lam, seed, it + 1 == n_steps);
+  if (rc == RW_OK) return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "train launch");
+  // the steps before the one that failed have changed the parameters
+  const std::string why = m->err;
+  refresh_wt(m);
+  m->err = why;
+  return rc;
 }
 
 int rw_mlp_set_gemm(rw_mlp* m, int kind) {

@@ -58,3 +58,27 @@ for device in (0, 1):
         assert train(m, 2) == 0 and forward(m) == 0, (device, gemm, lib.rw_mlp_last_error(m))
     lib.rw_mlp_destroy(m)
 """)
+
+
+def test_packed_weights_follow_the_parameters_after_a_failed_step(run):
+    """Whichever launch of a training run fails, the inference that follows packs or has packed the weights after the last
+    update of the parameters, and so have the transposes been made."""
+    run("""
+m = model(0)
+fake.fake_clear()
+assert train(m, 1) == 0
+step = kernels()
+assert step.count("k_adam") == 1 and step[-2:] == ["k_transpose_bf16", "k_pack_infer"], step
+for n in range(1, 3 * len(step)):
+    fake.fake_clear()
+    fake.fake_fail_launch(n)
+    rc = train(m, 3)
+    fake.fake_fail_launch(0)
+    assert rc == (-5 if n <= 3 * len(step) - 2 else 0), (n, rc)  # all but the last step leave the packing out
+    assert forward(m) == 0
+    log = kernels()
+    assert log[-1] == "k_mlp_infer", log
+    if "k_adam" in log:
+        after = log[len(log) - 1 - log[::-1].index("k_adam"):]
+        assert "k_transpose_bf16" in after and "k_pack_infer" in after, (n, after)
+""")
