@@ -7,10 +7,10 @@
 // Why: one thread (or one lane per helicity slice) per event repeats every
 // current for each helicity it does not depend on and spills; its unrolled code
 // overflows the instruction cache.  Here the sum takes about half the
-// arithmetic, the code is compact loops over tasks, and 8 (FP64) or 16 (FP32)
-// warps fit an SM.  FP64 is bound by the FP64 pipe (90 % busy), FP32 by issue,
-// instruction fetch and shared-memory latency (2.5 of 4 instructions per cycle
-// before its warps were kept in step).  Per call with one point, against the
+// arithmetic, the code is compact loops over tasks, and 8 (FP64) or 16 (FP32, 8
+// where the sums of 19 points or more take the room) warps fit an SM.  FP64 is
+// bound by the FP64 pipe (92 % busy), FP32 by issue (71 %), shared-memory
+// latency and addressing.  Per call with one point, against the
 // per-thread kernels: FP64 131,072 events 118 -> 53.1 ms (57.5 before products
 // of currents were shared between the three- and four-gluon currents), FP32
 // 262,147 events 15.3 -> 3.31 ms, FP16-mixed 65,536 events 3.94 -> 1.13 ms.

@@ -881,10 +881,14 @@ int backward_tc(rw_mlp* m, const float* y, int B, float inv_tau2, float lam) {
   return cudaGetLastError() == cudaSuccess ? RW_OK : mlp_fail(m, RW_ERR_CUDA, "backward launch");
 }
 
-// From 2,048 rows on: there a last-bit difference in a gradient's sum vanishes
-// in the average over the batch.  Below, it turns enough BF16 roundings in the
-// steps that follow to move the first moments by 2.6e-5 over 16 steps of 1,000
-// rows (7e-6 with 4,096), so small batches keep the row-by-row sums' order.
+// From 2,048 rows on.  Below, small batches keep the results they had: the sums'
+// other order turns BF16 roundings in the steps that follow, which moves the
+// first moments by 2.6e-5 over 16 steps of 1,000 rows (7e-6 with 4,096).  This
+// is not a bound on accuracy: against FP64 the two paths' gradients (40 -> 4 x
+// 256, 2-norm) are off by the same 3.05e-3 at 64 rows, 1.87e-3 at 512, 1.17e-3
+// at 1,000, 8.4e-4 at 2,000 and 3.1e-4 at 16,384, and a training step through
+// the tensor-core path would take 110 instead of 207 us at 64 rows, 140 instead
+// of 250 us at 1,000 (142 and 266 us at 2,048, 171 and 610 us at 16,384).
 constexpr int WG_MIN_ROWS = 2048;
 bool backward_tc_usable(const rw_mlp* m, int B) {
   return m->wparts && m->n_layers >= 2 && B >= WG_MIN_ROWS && tc_usable(m);

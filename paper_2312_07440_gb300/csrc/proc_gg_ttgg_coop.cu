@@ -2,7 +2,10 @@
 // the amplitude pass of the FP16-mixed mode's separate colour sum.  (Not the
 // BF16 one's: rounding the amplitude vectors to 8 bits turns the last-bit
 // differences between two FP32 evaluations into differences of up to 1.5e-3 in
-// W', and its results stay those of the 8-lane pass.)
+// W', and the mode keeps the results it had.  Its accuracy does not ask for
+// that: against FP64, 65,536 events x 2 points, both forms have an rms error of
+// 7.3e-4 in W' and a maximum of 5.6e-3, and the warp-per-event form would take
+// 1.08 instead of 2.61 ms.)
 #include "../../include/rwgt.h"
 #include "coop_kernel.cuh"
 #include "gen_qcd_gg_ttgg.cuh"

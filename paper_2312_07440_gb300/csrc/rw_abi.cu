@@ -72,8 +72,9 @@ int default_lane_bits(int process, int mode) {
     case RW_EE_MUMU: return 2;
     case RW_GG_TT: return 0;
     case RW_GG_TTG: return 0;
-    // the BF16-mixed amplitude pass has no warp-per-event form; 8 lanes beat 4
-    // (65,536 events, one point: 2.69 against 3.74 ms)
+    // the BF16-mixed amplitude pass keeps its per-thread form
+    // (proc_gg_ttgg_coop.cu); 8 lanes beat 4 (65,536 events, one point: 2.61
+    // against 3.67 ms)
     case RW_GG_TTGG: return mode == RW_MIXED_BF16 ? 3 : 5;
     case RW_EE_5A: return 0;
   }
@@ -355,7 +356,11 @@ bool block_chosen(const rw_ctx* c, const KernelEntry* k) {
 // The warp-per-event kernels (32 lanes) run 8 warps per block, 2 when there are
 // too few events to give every SM that many, which spreads them over the SMs;
 // and fewer than that, or than the caller's choice, where the sums of many
-// points leave no room for it: the points may be set after the choice.
+// points leave no room for it: the points may be set after the choice.  Sums
+// cost 24 bytes per point and warp: two FP32 blocks of 8 warps fit an SM up to
+// 18 points and one from 19 on (6.3 against 7.4 ns per event and evaluation at
+// 18 and at 64 distinct masses; the per-thread kernel takes 28.1); an FP64 block
+// has 8 warps up to 64 points and 4 from 65 on (205 against 199 ns; 742).
 int block_for(const rw_ctx* c, const KernelEntry* k, long long E, int npts) {
   const bool chosen = block_chosen(c, k);
   if (k->lane_bits < 5) return chosen ? c->block : 128;
