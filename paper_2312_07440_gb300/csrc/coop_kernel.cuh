@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_coop(const __gr
     if constexpr (!STORE) {
       __syncwarp();
       if (!valid) continue;
-      const double me0 = with_coupling(sums[0], a.pt[0].cscale);
+      const double me0 = with_coupling<true>(sums[0], a.pt[0].cscale);
       if (a.me_only) {
         if (lane == 0) a.me0[ev] = me0;
         continue;
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_coop(const __gr
       for (int j = lane; j <= P; j += 32) {
         double x = w;
         if (j < P) {
-          const double me = with_coupling(sums[a.kin_of[j + 1]], a.pt[j + 1].cscale);
+          const double me = with_coupling<true>(sums[a.kin_of[j + 1]], a.pt[j + 1].cscale);
           const double r = ok ? me / me0 : 0.0;
           x = ok ? r * w : 0.0;
           const long long o = (long long)j * ldo + ev;

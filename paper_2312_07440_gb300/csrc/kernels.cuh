@@ -191,9 +191,11 @@ __device__ __forceinline__ double eval_point(const typename Proc::template mom_t
 
 // |M|^2 from its coupling-stripped sum.  An event outside a point's phase space
 // (sum 0) has none, also where the coupling's power overflows: 0, not 0 x inf.
-// (The sum's bits are compared: an FP64 comparison takes the FP64 pipe.)
+// MOVES: whether the process moves events at all (the guard costs e+e- -> 5
+// photons FP32, 250,000 events x 8 couplings, 788 -> 798 us).
+template <bool MOVES>
 __device__ __forceinline__ double with_coupling(double s, double cscale) {
-  return (__double_as_longlong(s) << 1) != 0 ? s * cscale : 0.0;
+  return !MOVES || __double2hiint(cscale) != 0x7FF00000 || s != 0.0 ? s * cscale : 0.0;
 }
 
 // The end of a reweighting launch: the block's warp sums sacc [nwarps][P+1] to
@@ -335,13 +337,13 @@ __global__ void __launch_bounds__(256, MINB) k_reweight(const __grid_constant__ 
       else
         s = eval_point<Proc, R, LB>(p, pk, lane, gmask);
       if (a.me_only) {
-        if (leader) a.me0[ev] = with_coupling(s, a.pt[0].cscale);
+        if (leader) a.me0[ev] = with_coupling<Proc::MOVES>(s, a.pt[0].cscale);
         break;
       }
 #pragma unroll 1
       for (; at < a.kin_end[k]; ++at) {
         const int j = a.order[at];
-        const double me = with_coupling(s, a.pt[j].cscale);
+        const double me = with_coupling<Proc::MOVES>(s, a.pt[j].cscale);
         double contrib;
         if (j == 0) {
           me0 = me;

@@ -82,7 +82,7 @@ __device__ __forceinline__ void multi_tile(const MultiItem& a, const PointDev* p
   bool ok = false;
 #pragma unroll 1
   for (int j = 0; j <= P; ++j) {
-    const double me = with_coupling(eval_point<Proc, R, LB>(p, pts[a.pt0 + j], lane, gmask), pts[a.pt0 + j].cscale);
+    const double me = with_coupling<Proc::MOVES>(eval_point<Proc, R, LB>(p, pts[a.pt0 + j], lane, gmask), pts[a.pt0 + j].cscale);
     if (j == 0) {
       me0 = me;
       ok = isfinite(me0) && me0 != 0.0;

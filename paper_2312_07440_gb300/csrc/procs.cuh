@@ -31,6 +31,7 @@ template <class Tag, int CM = 0>
 struct QcdProc {
   static constexpr int NG = Tag::NG;
   static constexpr int NEXT = Tag::NEXT;
+  static constexpr bool MOVES = true;  // a new top mass moves the event, or does not fit it
   static constexpr int NCOL = Tag::NCOL;
   static constexpr bool kSymmetricHelicities = true;
   // per-event constants (external wavefunctions and propagator invariants):
@@ -152,6 +153,7 @@ template <class Tag>
 struct QedProc {
   static constexpr int NA = Tag::NA;
   static constexpr int NEXT = Tag::NEXT;
+  static constexpr bool MOVES = false;
   template <class R>
   using mom_t = typename std::conditional<sizeof(R) == 8, double, df>::type;
   template <class R, int LB = 0>
@@ -201,6 +203,7 @@ struct QedProc {
 // currents carry no parameter and are formed once per event (54 -> 45 us).
 struct EeMumu {
   static constexpr int NEXT = 4;
+  static constexpr bool MOVES = false;
   static constexpr int NHEL = 16;
   // FP64 momenta in every mode (a 4-particle process with no reshuffle: its
   // few FP64 invariants per event are not a bottleneck)
